@@ -69,8 +69,9 @@ typedef enum {
     HVOX_EINVAL = 1,        /* bad argument; nothing was enqueued */
     HVOX_ENOMEM = 2,        /* device or host allocation failed */
     HVOX_ECUDA = 3,         /* a CUDA runtime or cuFFT call failed */
-    HVOX_ETIMEOUT = 4,      /* reserved: no kernel of this library waits on a flag, a peer
-                               or another kernel, so no call returns it */
+    HVOX_ETIMEOUT = 4,      /* a direct-sum kernel's bounded wait inside its own pipeline (never on
+                               another kernel or a peer) ran out after ~2 s: reported like the
+                               device error word below; its outputs are NaN */
     HVOX_EUNSUPPORTED = 5,  /* option combination not supported */
     HVOX_EINTERNAL = 6      /* internal invariant violated; also the plan's device error
                                word: a kernel found a spreading or interpolation window
@@ -192,7 +193,8 @@ typedef struct {
     int32_t fft_batches;         /* batched FFTs of a transform (one per grid shape and wave) */
     int32_t fft_batches_df;      /* of those, FP64 grids transformed in double-float arithmetic
                                     on the FP32 pipes (the rest: cuFFT) */
-    int32_t direct_vpt;          /* owners (points) per thread of the direct kernels, 2 or 4 */
+    int32_t direct_vpt;          /* owners (points) per thread of the direct kernels: 1 on the tensor-
+                                    core forms (FP32, double-float), 2 on the FP64 form */
 } hvox_info;
 
 /*
@@ -351,8 +353,8 @@ const char *hvox_version(void);
  *   V interleaved complex float[2 n_vis] (overwritten): all DEVICE pointers (host
  *   pointers are rejected with HVOX_EINVAL). stream: cudaStream_t or NULL.
  * Limit: n_pix + n_vis <= 524,288 (HVOX_EINVAL beyond, nothing enqueued). The working
- * memory is one static device array of 16 MiB (coordinate splits), held on every GPU
- * that loads it until the process exits; the call itself calls no cudaMalloc, cudaFree
+ * memory is one static device array of 16 MiB and 16 bytes (coordinate splits), held on
+ * every GPU that loads it until the process exits; the call itself calls no cudaMalloc, cudaFree
  * or allocating library routine. CUDA loads device code lazily by default, so the array
  * is reserved on a device by the first call of this function there (or the first
  * direct-sum launch of any plan there): a caller whose framework will take the whole
@@ -361,9 +363,8 @@ const char *hvox_version(void);
  * array's device address (cudaGetSymbolAddress) with the device current; make that first
  * call before any stream capture. All calls share the array and it keeps the last call's
  * contents, so calls whose work overlaps on the GPU (different streams, or different
- * host threads) race: serialise them. The sum over pixels runs in segments of 4096
- * pixels whose partial sums meet through atomic adds, so the last bits of V may differ
- * between calls. Asynchronous on `stream`.
+ * host threads) race: serialise them. The sum over pixels runs in segments whose partial
+ * sums meet through atomic adds, so the last bits of V may differ between calls. Asynchronous on `stream`.
  */
 hvox_status hvox_direct_synthesize_noalloc(const double *pix_xyz, int64_t n_pix, const double *uvw, int64_t n_vis,
                                            const float *I, float *V, int isign, void *stream);

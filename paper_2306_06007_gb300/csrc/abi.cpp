@@ -126,6 +126,10 @@ void check_device_error(Plan &p) {
     check_cuda(cudaMemcpy(&word, p.err.ptr, sizeof(int), cudaMemcpyDeviceToHost), "read device error word");
     if (word == 0) return;
     check_cuda(cudaMemset(p.err.ptr, 0, sizeof(int)), "clear device error word");
+    if (word & kDevErrStall)
+        fail(HVOX_ETIMEOUT, "device error word " + std::to_string(word) +
+                                ": a direct-sum kernel's wait inside its pipeline ran out; the transforms since the last "
+                                "check are wrong");
     std::string what;
     if (word & kDevErrPixWindow) what += " a pixel window fell outside its sub-problem's n1 grid;";
     if (word & kDevErrVisWindow) what += " a baseline window fell beyond one period of its n2 grid;";
@@ -207,18 +211,18 @@ void upload(DevBuf &b, const void *host, size_t bytes, cudaStream_t s) {
     if (bytes) check_cuda(cudaMemcpyAsync(b.ptr, host, bytes, cudaMemcpyHostToDevice, s), "upload");
 }
 
-void build_items(const std::vector<DirectRect> &rects, bool owner_is_vis, int vpt, std::vector<WorkItem> &items) {
-    const int64_t T = direct_tile(vpt);
+void build_items(const std::vector<DirectRect> &rects, bool owner_is_vis, int kind, std::vector<WorkItem> &items) {
+    const int64_t T = direct_tile(kind);
+    // One rectangle (most jobs): segments that come out evenly. Many: about 32 items per SM in
+    // all, taken dynamically by the kernels largest first, so that a launch ends within a fraction
+    // of an item of its ideal time.
     double work = 0;
     for (auto &r : rects) work += (double)(r.p1 - r.p0) * (double)(r.v1 - r.v0);
-    // About 32 items per resident CTA (152 SMs x 4), taken dynamically by the kernels
-    // largest first: a launch then ends within a fraction of an item of its ideal time.
-    const double target_items = 152.0 * 4.0 * 32.0;
-    int64_t seg = (int64_t)std::ceil(work / ((double)T * target_items) / 256.0) * 256;
-    seg = std::max<int64_t>(seg, 2048);
+    const int64_t even = std::max<int64_t>(2048, (int64_t)std::ceil(work / ((double)T * 152.0 * 32.0) / 256.0) * 256);
     for (auto &r : rects) {
         int64_t o0 = owner_is_vis ? r.v0 : r.p0, o1 = owner_is_vis ? r.v1 : r.p1;
         int64_t s0 = owner_is_vis ? r.p0 : r.v0, s1 = owner_is_vis ? r.p1 : r.v1;
+        const int64_t seg = rects.size() == 1 ? direct_segment((o1 - o0 + T - 1) / T, s1 - s0) : even;
         for (int64_t o = o0; o < o1; o += T)
             for (int64_t q = s0; q < s1; q += seg)
                 items.push_back(WorkItem{(int32_t)o, (int32_t)std::min(o + T, o1), (int32_t)q,
@@ -442,9 +446,17 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
 
     // Direct work lists.
     {
+        float top = 0.f;
+        for (double v : pix) top = std::max(top, std::fabs((float)v));
+        coord_scales(top, p.pix_scale, p.vis_scale);
+        float far = 0.f;
+        for (double v : uvw) far = std::max(far, std::fabs((float)v));
+        far *= p.vis_scale;
+        if (p.direct_kind == kDirectF32 && !(far <= kF32Reach)) p.direct_kind = kDirectWide;
+        if (p.direct_kind == kDirectDf && !(far <= kDfReach)) p.direct_kind = kDirectF64;
         std::vector<WorkItem> a, b;
-        build_items(part.rects, true, p.direct_vpt, a);
-        build_items(part.rects, false, p.direct_vpt, b);
+        build_items(part.rects, true, p.direct_kind, a);
+        build_items(part.rects, false, p.direct_kind, b);
         p.item_counter.alloc(2 * sizeof(int));
         p.err.alloc(sizeof(int));
         check_cuda(cudaMemsetAsync(p.err.ptr, 0, sizeof(int), s), "clear device error word");
@@ -787,12 +799,7 @@ void configure(Plan &p, int64_t n_pix, int64_t n_vis, double eps, int isign, con
     // keeps FP64 shared atomics (comparisons).
     p.int_tile = p.prec == 2 && !p.plain;
     if (const char *v = std::getenv("HVOX_SPREAD_TILE")) p.int_tile = p.int_tile && std::string(v) != "float";
-    // Owners per thread of the direct kernels: four for the double-float kernels (LOFAR-like
-    // sky x 1.4M baselines at eps 1e-9: 320.2 against 327.8 ms per step), two for the FP32
-    // ones (config 2 at eps 1e-6: 125.3 against 126.8 ms) and the FP64 ones. HVOX_DIRECT_VPT
-    // (2 or 4) overrides.
-    p.direct_vpt = (p.prec == 2 && !p.direct_f64) ? 4 : 2;
-    if (const char *v = std::getenv("HVOX_DIRECT_VPT")) p.direct_vpt = std::atoi(v) == 4 ? 4 : 2;
+    p.direct_kind = p.direct_f64 ? kDirectF64 : p.prec == 1 ? kDirectF32 : kDirectDf;
 }
 
 void fill_info(const Plan &p, hvox_info *info) {
@@ -832,7 +839,7 @@ void fill_info(const Plan &p, hvox_info *info) {
     info->spread_bin_vis = p.ppc_vis;
     info->kernel_width_rule = es_params_within(p.eps_es, p.eps > 0 ? p.eps : 1e-6, p.sigma).w;
     info->probe_error = p.probe_error;
-    info->direct_vpt = p.direct_vpt;
+    info->direct_vpt = direct_owners_per_thread(p.direct_kind);
     info->fft_batches = info->fft_batches_df = 0;
     for (const Wave &w : p.waves)
         for (const FftBatch &f : w.ffts) {

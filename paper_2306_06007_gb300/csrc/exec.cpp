@@ -145,6 +145,30 @@ void run_waves(Plan &p, int dir, const In *src, Out *acc, cudaStream_t s, Profil
     }
 }
 
+// The plan as a job of the direct kernels.
+DirectJob job_of_plan(const Plan &p, int dir) {
+    const float4 *ph = p.pix_hi.as<float4>(), *pl = p.pix_lo.as<float4>();
+    const float4 *vh = p.vis_hi.as<float4>(), *vl = p.vis_lo.as<float4>();
+    if (dir == 0) return {vh, vl, ph, pl, p.src.ptr, p.acc.ptr, (float)p.isign, p.pix_scale, p.vis_scale, p.err.as<int>()};
+    return {ph, pl, vh, vl, p.src.ptr, p.acc.ptr, (float)p.isign, p.pix_scale, p.vis_scale, p.err.as<int>()};
+}
+
+// The direct sums of one plan in a launch of their own.
+void run_direct(Plan &p, int dir, cudaStream_t s) {
+    const WorkItem *it = (dir == 0 ? p.items_s2v : p.items_v2s).as<WorkItem>();
+    const int64_t n = dir == 0 ? p.n_items_s2v : p.n_items_v2s;
+    int *counter = p.item_counter.as<int>() + dir;
+    check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset item counter");
+    if (p.direct_kind != kDirectF64)
+        launch_direct(p.direct_kind, dir, it, n, counter, job_of_plan(p, dir), p.cis_tab.as<float4>(), s);
+    else if (dir == 0)
+        launch_direct_s2v_f64(it, n, counter, p.vis_xyz.as<double>(), p.n_vis, p.pix_xyz.as<double>(), p.n_pix,
+                              p.src.as<double>(), p.acc.as<double2>(), p.isign, s);
+    else
+        launch_direct_v2s_f64(it, n, counter, p.pix_xyz.as<double>(), p.n_pix, p.vis_xyz.as<double>(), p.n_vis,
+                              p.src.as<double2>(), p.acc.as<double>(), p.isign, s);
+}
+
 // sky -> vis between the permutations: src (chunk-ordered c_n) -> acc (chunk-ordered V).
 void body_s2v(Plan &p, cudaStream_t s, Profiler &prof) {
     const size_t re = real_bytes(p);
@@ -154,20 +178,7 @@ void body_s2v(Plan &p, cudaStream_t s, Profiler &prof) {
     fork_lanes(p, s);
     if (p.n_items_s2v > 0) {
         prof.begin(HVOX_STAGE_DIRECT, s);
-        const WorkItem *it = p.items_s2v.as<WorkItem>();
-        int *counter = p.item_counter.as<int>();
-        check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset item counter");
-        if (p.direct_f64)
-            launch_direct_s2v_f64(it, p.n_items_s2v, counter, p.vis_xyz.as<double>(), p.n_vis, p.pix_xyz.as<double>(),
-                                  p.n_pix, p.src.as<double>(), p.acc.as<double2>(), p.isign, p.direct_vpt, s);
-        else if (p.prec == 1)
-            launch_direct_s2v_f32(it, p.n_items_s2v, counter, p.vis_hi.as<float4>(), p.vis_lo.as<float4>(),
-                                  p.pix_hi.as<float4>(), p.pix_lo.as<float4>(), p.src.as<float>(),
-                                  p.acc.as<float2>(), p.isign, p.direct_vpt, s);
-        else
-            launch_direct_s2v_df(it, p.n_items_s2v, counter, p.vis_hi.as<float4>(), p.vis_lo.as<float4>(),
-                                 p.pix_hi.as<float4>(), p.pix_lo.as<float4>(), p.src.as<double>(),
-                                 p.acc.as<double2>(), p.cis_tab.as<float4>(), p.isign, p.direct_vpt, s);
+        run_direct(p, 0, s);
         prof.end(HVOX_STAGE_DIRECT, 1, s);
     }
     if (!p.waves.empty()) {
@@ -188,20 +199,7 @@ void body_v2s(Plan &p, cudaStream_t s, Profiler &prof) {
     fork_lanes(p, s);
     if (p.n_items_v2s > 0) {
         prof.begin(HVOX_STAGE_DIRECT, s);
-        const WorkItem *it = p.items_v2s.as<WorkItem>();
-        int *counter = p.item_counter.as<int>() + 1;
-        check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset item counter");
-        if (p.direct_f64)
-            launch_direct_v2s_f64(it, p.n_items_v2s, counter, p.pix_xyz.as<double>(), p.n_pix, p.vis_xyz.as<double>(),
-                                  p.n_vis, p.src.as<double2>(), p.acc.as<double>(), p.isign, p.direct_vpt, s);
-        else if (p.prec == 1)
-            launch_direct_v2s_f32(it, p.n_items_v2s, counter, p.pix_hi.as<float4>(), p.pix_lo.as<float4>(),
-                                  p.vis_hi.as<float4>(), p.vis_lo.as<float4>(), p.src.as<float2>(),
-                                  p.acc.as<float>(), p.isign, p.direct_vpt, s);
-        else
-            launch_direct_v2s_df(it, p.n_items_v2s, counter, p.pix_hi.as<float4>(), p.pix_lo.as<float4>(),
-                                 p.vis_hi.as<float4>(), p.vis_lo.as<float4>(), p.src.as<double2>(),
-                                 p.acc.as<double>(), p.cis_tab.as<float4>(), p.isign, p.direct_vpt, s);
+        run_direct(p, 1, s);
         prof.end(HVOX_STAGE_DIRECT, 1, s);
     }
     if (!p.waves.empty()) {
@@ -368,51 +366,13 @@ namespace {
 
 // The direct sums of one plan alone (FP64 kernels, or any plan outside a merged launch).
 void direct_alone(Plan &p, int dir, cudaStream_t s) {
-    const int64_t n = dir == 0 ? p.n_items_s2v : p.n_items_v2s;
-    if (n <= 0) return;
-    const WorkItem *it = (dir == 0 ? p.items_s2v : p.items_v2s).as<WorkItem>();
-    int *counter = p.item_counter.as<int>() + dir;
-    check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset item counter");
-    if (dir == 0) {
-        if (p.direct_f64)
-            launch_direct_s2v_f64(it, n, counter, p.vis_xyz.as<double>(), p.n_vis, p.pix_xyz.as<double>(), p.n_pix,
-                                  p.src.as<double>(), p.acc.as<double2>(), p.isign, p.direct_vpt, s);
-        else if (p.prec == 1)
-            launch_direct_s2v_f32(it, n, counter, p.vis_hi.as<float4>(), p.vis_lo.as<float4>(), p.pix_hi.as<float4>(),
-                                  p.pix_lo.as<float4>(), p.src.as<float>(), p.acc.as<float2>(), p.isign,
-                                  p.direct_vpt, s);
-        else
-            launch_direct_s2v_df(it, n, counter, p.vis_hi.as<float4>(), p.vis_lo.as<float4>(), p.pix_hi.as<float4>(),
-                                 p.pix_lo.as<float4>(), p.src.as<double>(), p.acc.as<double2>(),
-                                 p.cis_tab.as<float4>(), p.isign, p.direct_vpt, s);
-    } else {
-        if (p.direct_f64)
-            launch_direct_v2s_f64(it, n, counter, p.pix_xyz.as<double>(), p.n_pix, p.vis_xyz.as<double>(), p.n_vis,
-                                  p.src.as<double2>(), p.acc.as<double>(), p.isign, p.direct_vpt, s);
-        else if (p.prec == 1)
-            launch_direct_v2s_f32(it, n, counter, p.pix_hi.as<float4>(), p.pix_lo.as<float4>(), p.vis_hi.as<float4>(),
-                                  p.vis_lo.as<float4>(), p.src.as<float2>(), p.acc.as<float>(), p.isign,
-                                  p.direct_vpt, s);
-        else
-            launch_direct_v2s_df(it, n, counter, p.pix_hi.as<float4>(), p.pix_lo.as<float4>(), p.vis_hi.as<float4>(),
-                                 p.vis_lo.as<float4>(), p.src.as<double2>(), p.acc.as<double>(),
-                                 p.cis_tab.as<float4>(), p.isign, p.direct_vpt, s);
-    }
+    if ((dir == 0 ? p.n_items_s2v : p.n_items_v2s) <= 0) return;
+    run_direct(p, dir, s);
     p.stage_launches[HVOX_STAGE_DIRECT] += 1;
 }
 
-// The job of a plan in a merged direct launch.
-DirectJob job_of_plan(const Plan &p, int dir) {
-    if (dir == 0)
-        return {p.vis_hi.as<float4>(), p.vis_lo.as<float4>(), p.pix_hi.as<float4>(), p.pix_lo.as<float4>(),
-                p.src.ptr,             p.acc.ptr,             (float)p.isign};
-    return {p.pix_hi.as<float4>(), p.pix_lo.as<float4>(), p.vis_hi.as<float4>(), p.vis_lo.as<float4>(),
-            p.src.ptr,             p.acc.ptr,             (float)p.isign};
-}
-
-// One merged launch over the work items of the plans in `group` (same kernel form and
-// owners per thread). Its lists live in one stream-ordered allocation freed after it.
-void direct_merged(const std::vector<Plan *> &group, int dir, int kind, int vpt, cudaStream_t s) {
+// One merged launch over the work items of the plans in `group` (same kernel form). Its lists live in one stream-ordered allocation freed after it.
+void direct_merged(const std::vector<Plan *> &group, int dir, int kind, cudaStream_t s) {
     std::vector<DirectJob> jobs;
     std::vector<std::pair<int64_t, int>> order;  // (pairs, index into flat) for the sort
     std::vector<WorkItem> flat;
@@ -449,7 +409,7 @@ void direct_merged(const std::vector<Plan *> &group, int dir, int kind, int vpt,
     check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset batch counter");
     launch_direct_batch(kind, dir, reinterpret_cast<const WorkItem *>(d), n, counter,
                         reinterpret_cast<const DirectJob *>(d + up(b_items) + up(b_job)),
-                        reinterpret_cast<const int *>(d + up(b_items)), group[0]->cis_tab.as<float4>(), vpt, s);
+                        reinterpret_cast<const int *>(d + up(b_items)), group[0]->cis_tab.as<float4>(), s);
     check_cuda(cudaFreeAsync(dev, s), "cudaFreeAsync (batch work list)");
     for (Plan *p : group) p->stage_launches[HVOX_STAGE_DIRECT] += 1;
 }
@@ -482,23 +442,23 @@ int run_batch(const std::vector<Plan *> &plans, const std::vector<const void *> 
         p.stage_launches[HVOX_STAGE_ZERO] += 1;
         fork_lanes(p, s);
     }
-    // direct sums: merged per (kernel form, owners per thread); FP64 kernels alone
+    // direct sums: merged per kernel form; FP64 kernels alone
     int launches = 0;
-    std::map<std::pair<int, int>, std::vector<Plan *>> groups;
+    std::map<int, std::vector<Plan *>> groups;
     for (Plan *p : plans) {
         if ((dir == 0 ? p->n_items_s2v : p->n_items_v2s) <= 0) continue;
-        if (p->direct_f64) {
+        if (p->direct_kind == kDirectF64) {
             direct_alone(*p, dir, s);
             ++launches;
         } else {
-            groups[{p->prec == 1 ? 0 : 1, p->direct_vpt}].push_back(p);
+            groups[p->direct_kind].push_back(p);
         }
     }
     for (auto &g : groups) {
         if (g.second.size() == 1)
             direct_alone(*g.second[0], dir, s);
         else
-            direct_merged(g.second, dir, g.first.first, g.first.second, s);
+            direct_merged(g.second, dir, g.first, s);
         ++launches;
     }
     // NUFFT sub-problems on each plan's lanes, outputs back to the callers' order

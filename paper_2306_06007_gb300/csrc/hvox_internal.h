@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <cufft.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <map>
 #include <memory>
@@ -45,7 +47,8 @@ bool fault_hit(const char *site);
 // Bits of a plan's device error word, set by kernels that had to clamp an index.
 enum : int {
     kDevErrPixWindow = 1,   // a pixel window outside the n1 grid (clamped into it)
-    kDevErrVisWindow = 2    // a baseline window beyond one period of the n2 grid (clamped)
+    kDevErrVisWindow = 2,   // a baseline window beyond one period of the n2 grid (clamped)
+    kDevErrStall = 4        // a direct-sum kernel's bounded wait inside its pipeline ran out
 };
 
 // ------------------------------------------------------------------ ES kernel
@@ -105,14 +108,59 @@ struct WorkItem {
 
 // Device pointers of one job of a direct launch (one plan's chunk-ordered buffers): owner
 // coordinates (sky -> vis: baselines, vis -> sky: pixels) and streamed coordinates as
-// hi / lo float4 splits, the streamed values (c or V), the owners' accumulators, and the
-// exponent's sign.
+// hi / lo float4 splits, the streamed values (c or V), the owners' accumulators, the
+// exponent's sign, and the powers of two that bring pixel coordinates into [-1, 1]
+// (pix_scale) and leave every product with a baseline as it was (vis_scale = 1 / pix_scale).
 struct DirectJob {
     const float4 *own_hi, *own_lo, *str_hi, *str_lo;
     const void *val;
     void *acc;
     float sgn;
+    float pix_scale, vis_scale;
+    int *err;  // the plan's device error word (may be null)
 };
+
+// The two powers of two for pixels of largest |coordinate| top (1 for unit vectors).
+__host__ __device__ inline void coord_scales(float top, float &pix_scale, float &vis_scale) {
+    int e = 0;
+    if (top > 0.f) frexpf(top, &e);         // top = f 2^e, 1/2 <= f < 1
+    if (top == ldexpf(1.f, e - 1)) --e;     // a power of two is its own bound
+    e = e < -60 ? -60 : e > 60 ? 60 : e;
+    pix_scale = ldexpf(1.f, -e);
+    vis_scale = ldexpf(1.f, e);
+}
+
+// Forms of the direct kernels.
+enum { kDirectF32 = 0, kDirectDf = 1, kDirectF64 = 2, kDirectWide = 3 };
+
+// Largest |p_d| times pixel scale (turns per dimension) that the digits of each form reach: an
+// FP32 plan beyond its reach runs the double-float form on its float values, a double-float
+// one the FP64 kernels.
+constexpr float kF32Reach = 0x1p28f, kDfReach = 0x1p33f;
+
+// Streamed points per work item for a rectangle of `tiles` owner tiles x `n` streamed points,
+// a multiple of 64 chosen so that the items come out evenly over `slots` CTAs: the segment
+// count s of least modelled time, ceil(tiles s / slots) rounds of one segment and an item's
+// fixed cost of about 128 streamed points (owners' digits, pipeline fill, output atomics). A
+// fixed segment of 2,048 left a 1,000 x 1,000 request with two items for 152 SMs, and one of
+// 256 points cost a third more than its sums. Segments meet in FP32 atomics, whose rounding
+// grows with their number, so there are at most 32 or one per 2,048 points, or as many as
+// fill the slots once.
+inline int64_t direct_segment(int64_t tiles, int64_t n, int64_t slots = 152) {
+    const int64_t most = std::max<int64_t>({32, (n + 2047) / 2048, (slots + tiles - 1) / tiles});
+    int64_t best = 0;
+    double best_cost = 0.0;
+    for (int64_t s = 1; s <= most; ++s) {
+        const int64_t seg = ((n + s - 1) / s + 63) / 64 * 64;
+        const int64_t items = tiles * ((n + seg - 1) / seg);
+        const double cost = (double)((items + slots - 1) / slots) * (double)(seg + 128);
+        if (best == 0 || cost < best_cost) {
+            best = seg;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
 
 struct CostModel {
     double direct_pair = 0;      // seconds per (pixel, baseline) pair, one direction
@@ -343,7 +391,8 @@ struct Plan {
     bool plain = false;
     bool direct_f64 = false;       // direct sums by the FP64 kernels (plain form, or eps < 1e-9)
     int ntrans = 1;
-    int direct_vpt = 2;            // points per thread of the direct kernels (owner tile 256 * vpt)
+    int direct_kind = 0;           // kDirectF32, ...
+    float pix_scale = 1.f, vis_scale = 1.f;  // coord_scales of the pixels
     double sigma = 2.0;
     double budget_opt = 0.0;       // chunk_budget_bytes option (0 -> cost-model search)
     bool sigma_auto = true;        // upsampling chosen by the planner
@@ -418,25 +467,19 @@ void launch_prepare_points(const double *xyz_orig_dev, const int32_t *perm, int6
 void launch_gather_weight(const double *w_orig_dev, const int32_t *perm, int64_t n, double *w_perm,
                           cudaStream_t s);
 
-// Direct kernels (k_direct.cu). Owner tile = direct_tile() points per work item.
-int direct_tile(int vpt);
-void launch_direct_s2v_f32(const WorkItem *items, int64_t n, int *counter, const float4 *vh, const float4 *vl, const float4 *rh,
-                           const float4 *rl, const float *c, float2 *acc, int isign, int vpt, cudaStream_t s);
-void launch_direct_s2v_df(const WorkItem *items, int64_t n, int *counter, const float4 *vh, const float4 *vl, const float4 *rh,
-                          const float4 *rl, const double *c, double2 *acc, const float4 *tab, int isign,
-                          int vpt, cudaStream_t s);
-void launch_direct_s2v_f64(const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv, const double *pxyz,
-                           int64_t np, const double *c, double2 *acc, int isign, int vpt, cudaStream_t s);
-void launch_direct_v2s_f32(const WorkItem *items, int64_t n, int *counter, const float4 *rh, const float4 *rl, const float4 *vh,
-                           const float4 *vl, const float2 *V, float *acc, int isign, int vpt, cudaStream_t s);
-void launch_direct_v2s_df(const WorkItem *items, int64_t n, int *counter, const float4 *rh, const float4 *rl, const float4 *vh,
-                          const float4 *vl, const double2 *V, double *acc, const float4 *tab, int isign,
-                          int vpt, cudaStream_t s);
-void launch_direct_v2s_f64(const WorkItem *items, int64_t n, int *counter, const double *pxyz, int64_t np, const double *vxyz,
-                           int64_t nv, const double2 *V, double *acc, int isign, int vpt, cudaStream_t s);
-// Several jobs' items in one launch: kind 0 FP32, 1 double-float; dir 0 sky -> vis, 1 vis -> sky.
+// Direct kernels (k_direct.cu): owner points per work item and per thread, one job's launch
+// (any kind but FP64; dir 0 sky -> vis, 1 vis -> sky; counter zero at launch; tab the
+// 2048-entry table of exp(j 2 pi m / 2048), double-float only), and several jobs' items in one.
+int direct_tile(int kind);
+int direct_owners_per_thread(int kind);
+void launch_direct(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob &J,
+                   const float4 *tab, cudaStream_t s);
 void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob *jobs,
-                         const int *item_job, const float4 *tab, int vpt, cudaStream_t s);
+                         const int *item_job, const float4 *tab, cudaStream_t s);
+void launch_direct_s2v_f64(const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
+                           const double *pxyz, int64_t np, const double *c, double2 *acc, int isign, cudaStream_t s);
+void launch_direct_v2s_f64(const WorkItem *items, int64_t n, int *counter, const double *pxyz, int64_t np,
+                           const double *vxyz, int64_t nv, const double2 *V, double *acc, int isign, cudaStream_t s);
 
 // NUFFT sub-problems, one wave at a time (k_nufft.cu). g1 / g2: the lane's grid buffers.
 template <typename T>

@@ -5,21 +5,31 @@
 //   vis -> sky:  I_n += Re sum_k V_k exp(-isign j 2 pi <p_k, r_n>)
 //
 // The phase <p, r> reaches ~1e5 turns, so it is never formed in plain FP32. Every
-// coordinate is stored as a pair of floats hi + lo (hi = fl32(x), lo = fl32(x - hi)).
-// Per pair the main products hi(p) hi(r) are split exactly (TwoProduct by fma), their
-// integer turns dropped exactly, and only the fraction of a turn is carried on:
-//  * FP32 path (eps >= 1e-6): fraction in FP32 (abs error ~1e-7 turn), hardware
-//    sin/cos approximations, FP32 accumulation;
-//  * double-float path (eps < 1e-6): fraction as an unevaluated float pair; exp(j 2 pi f)
-//    as the hi parts of a periodic 2048-entry table of exp(j 2 pi m / 2048) plus a lo part
-//    (the table's lo parts and a short series in the remainder, in plain float; error
-//    2.7e-10); products and sums in double-float arithmetic (Dekker 1971);
-//  * plain path: everything in FP64 (the reference form the optimised paths replace).
+// coordinate is stored as a pair of floats hi + lo (hi = fl32(x), lo = fl32(x - hi)), and the
+// tensor cores form the turns modulo one of a tile of pairs from their digits (phase_tc.cuh):
+//  * FP32 path (eps >= 1e-6): fraction in FP32 (error ~1.5e-8 turn rms), hardware sin/cos
+//    approximations, FP32 accumulation;
+//  * double-float path (eps < 1e-6): exp(j 2 pi f) as the hi parts of a 1024-entry table of
+//    exp(j 2 pi m / 1024) plus a lo part (the table's lo parts and a short series in the
+//    remainder, in plain float; error ~1e-10); sums in double-float arithmetic (Dekker 1971);
+//  * wide path: the double-float path on the values of an FP32 plan whose |p_d r_d| exceed 2^28
+//    turns (the reach of the FP32 digits);
+//  * plain path: everything in FP64 (the reference form the optimised paths replace; also for
+//    |p_d r_d| above 2^33 turns).
+//
+// What bounds them: FP32 issue. A pair takes ~14 instructions at FP32 (2 on the sine unit at a
+// quarter rate, a bound of 16 cycles for 32 pairs) and ~42 in double-float (28 before and 73
+// before with the phase on the FP32 pipes). Measured on one GB300 over 52,812 pixels x 1,435,200
+// baselines: 1.9e12 pairs/s at FP32 (1.16e12 before) and 7.0e11 in double-float (4.7e11 before).
+#include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "hvox_internal.h"
+#include "phase_tc.cuh"
 
 namespace hvox {
 
@@ -27,7 +37,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kPerThread = 2;
-constexpr int kTile = kThreads * kPerThread;  // owner points per work item
+constexpr int kTile = kThreads * kPerThread;  // owner points per work item of the FP64 kernels
 
 // ------------------------------------------------------------- point preparation
 
@@ -66,115 +76,6 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &
     e = __fsub_rn(b, __fsub_rn(s, a));
 }
 
-__device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
-    p = __fmul_rn(a, b);
-    e = __fmaf_rn(a, b, -p);
-}
-
-// Round to nearest integer on the FMA pipe: adding and subtracting 1.5 * 2^23 leaves the
-// integer part for |x| < 2^22 (rintf would use the XU pipe, which the sin/cos need).
-constexpr float kRoundMagic = 12582912.0f;
-
-__device__ __forceinline__ float round_fma(float x) { return __fsub_rn(__fadd_rn(x, kRoundMagic), kRoundMagic); }
-
-// x - nearest integer, exact (the difference of a float and its rounding is exact).
-__device__ __forceinline__ float frac_fma(float x) { return __fsub_rn(x, round_fma(x)); }
-
-// Fraction of hi(p) hi(r) in turns for one dimension, in three FMA-pipe instructions:
-// t = fl(p r + 1.5 * 2^23) carries n = round(p r) exactly (float spacing 1 there, for
-// |p r| < 2^22), and fma(p, r, -n) forms the exact p r - n (|.| <= 1/2) with one rounding
-// (<= 2^-25 turn).
-__device__ __forceinline__ float prod_frac(float p, float r) {
-    const float n = __fsub_rn(__fmaf_rn(p, r, kRoundMagic), kRoundMagic);
-    return __fmaf_rn(p, r, -n);
-}
-
-// Fraction of <p, r> in turns, FP32 (|error| ~ 1e-7 turn), result in [-0.5, 0.5].
-// Valid for |p_d r_d| < 2^22 turns per dimension.
-__device__ __forceinline__ float phase_f32(const float3 &ph, const float3 &pl, const float4 &rh, const float4 &rl) {
-    float small = __fmaf_rn(ph.x, rl.x, __fmul_rn(pl.x, rh.x));
-    small = __fmaf_rn(ph.y, rl.y, __fmaf_rn(pl.y, rh.y, small));
-    small = __fmaf_rn(ph.z, rl.z, __fmaf_rn(pl.z, rh.z, small));
-    const float f = __fadd_rn(__fadd_rn(prod_frac(ph.x, rh.x), prod_frac(ph.y, rh.y)),
-                              __fadd_rn(prod_frac(ph.z, rh.z), small));
-    return frac_fma(f);
-}
-
-// Fraction of <p, r> in turns as an unevaluated float pair fh + fl with |fh| < 2
-// (integer turns dropped exactly per dimension; the sum of the three fractions is kept
-// exact with TwoSum), |error| ~ 1e-12 turn * |p| / 1e5.
-__device__ __forceinline__ void phase_df(const float3 &ph, const float3 &pl, const float4 &rh, const float4 &rl,
-                                         float &fh, float &fl) {
-    float a0, b0, a1, b1, a2, b2;
-    two_prod(ph.x, rh.x, a0, b0);
-    two_prod(ph.y, rh.y, a1, b1);
-    two_prod(ph.z, rh.z, a2, b2);
-    a0 = __fsub_rn(a0, rintf(a0));
-    a1 = __fsub_rn(a1, rintf(a1));
-    a2 = __fsub_rn(a2, rintf(a2));
-    float s1, e1, s2, e2;
-    two_sum(a0, a1, s1, e1);
-    two_sum(s1, a2, s2, e2);
-    float small = __fadd_rn(__fadd_rn(b0, b1), __fadd_rn(b2, __fadd_rn(e1, e2)));
-    small = __fmaf_rn(ph.x, rl.x, __fmaf_rn(pl.x, rh.x, small));
-    small = __fmaf_rn(ph.y, rl.y, __fmaf_rn(pl.y, rh.y, small));
-    small = __fmaf_rn(ph.z, rl.z, __fmaf_rn(pl.z, rh.z, small));
-    fast_two_sum(s2, small, fh, fl);
-}
-
-constexpr int kTabN = 2048;    // table entries per turn; the table is periodic in m
-
-// exp(j 2 pi f) for f = fh + fl (turns, |fh| < 1024) as re = reh + rel, im = imh + iml.
-// (reh, imh) are the hi parts of cos and sin of 2 pi m / 2048 for m = round(2048 fh), read
-// from T[m mod 2048] = (cos_h, cos_l, sin_h, sin_l). (rel, iml) collect the table's lo
-// parts and the rotation by x = 2 pi (fh - m/2048 + fl), |x| <= pi/2048, through
-// cos x - 1 = -x^2/2 and sin x = x - x^3/6 (dropped terms below 3e-13). Every term of a lo
-// part is below 1.6e-3 in magnitude, so plain float arithmetic keeps the pair within
-// ~2.5e-10 of exp(j 2 pi f); the hi parts need no error-free transformations.
-__device__ __forceinline__ void cis_tab(float fh, float fl, const float4 *__restrict__ T, float &reh, float &rel,
-                                        float &imh, float &iml) {
-    const float t = __fmaf_rn(fh, (float)kTabN, kRoundMagic);  // 1.5 * 2^23 + m
-    const int idx = __float_as_int(t) & (kTabN - 1);           // m mod 2048 (the magic's low bits are 0)
-    const float d = __fmaf_rn(__fsub_rn(t, kRoundMagic), -1.0f / kTabN, fh);  // fh - m/2048, exact
-    const float x = __fmul_rn(__fadd_rn(d, fl), 6.28318530717958648f);
-    const float x2 = __fmul_rn(x, x);
-    const float cm = __fmul_rn(x2, -0.5f);
-    const float sx = __fmaf_rn(__fmul_rn(x2, x), -1.0f / 6.0f, x);
-    const float4 tb = T[idx];
-    reh = tb.x;
-    rel = __fmaf_rn(-tb.z, sx, __fmaf_rn(tb.x, cm, tb.y));
-    imh = tb.z;
-    iml = __fmaf_rn(tb.x, sx, __fmaf_rn(tb.z, cm, tb.w));
-}
-
-__device__ __forceinline__ void df_mul(float ah, float al, float bh, float bl, float &ph, float &pl) {
-    float p, e;
-    two_prod(ah, bh, p, e);
-    e = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, e));
-    ph = p;
-    pl = e;
-}
-
-// Lazy double-float accumulation: hi carries an exact TwoSum, lo collects the errors.
-__device__ __forceinline__ void df_acc(float &acc_h, float &acc_l, float th, float tl) {
-    float s, e;
-    two_sum(acc_h, th, s, e);
-    acc_h = s;
-    acc_l = __fadd_rn(acc_l, __fadd_rn(e, tl));
-}
-
-// Offset double-float accumulation of one streamed tile: the running high sum starts at a
-// power of two M above twice the tile's sum of term magnitudes S, so it stays in
-// [M - S, M + S], never below any term, and the rounding error of each add is recovered
-// exactly by Fast2Sum (three instructions instead of TwoSum's six). The low part collects
-// those errors and the terms' own low parts. At the tile's end hi - M is exact (Sterbenz).
-__device__ __forceinline__ void df_acc_off(float &acc_h, float &acc_l, float th, float tl) {
-    const float s = __fadd_rn(acc_h, th);
-    const float e = __fsub_rn(th, __fsub_rn(s, acc_h));
-    acc_h = s;
-    acc_l = __fadd_rn(acc_l, __fadd_rn(e, tl));
-}
-
 // The offset for a tile whose term magnitudes sum to at most S: 2^(floor(log2 S) + 2) > 2 S
 // (S from the block's own values; tiny or zero S gives 2^-100).
 __device__ __forceinline__ float tile_offset(float S) {
@@ -182,22 +83,9 @@ __device__ __forceinline__ float tile_offset(float S) {
     return __uint_as_float(e + (2u << 23));
 }
 
-// Sum of x over the CTA (every thread gets it). red holds one float per warp; the caller
-// has a __syncthreads() between this call and the previous use of red.
-__device__ __forceinline__ float block_sum(float x, float *red) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
-    __syncthreads();
-    float t = 0.f;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) t += red[w];
-    return t;
-}
-
 // Kahan-compensated accumulation of per-tile partial sums: the FP32 paths sum each
-// 256-term shared-memory tile in registers and add the tile sums here, which keeps the
-// rounding error of sums over millions of terms near that of a 256-term sum.
+// thread's terms of a tile in registers and add the tile sums here, which keeps the
+// rounding error of sums over millions of terms near that of a short sum.
 __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x) {
     const float y = __fsub_rn(x, comp);
     const float t = __fadd_rn(sum, y);
@@ -206,8 +94,8 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x) {
 }
 
 // Adds a tile's double-float partial sum (ih + il) into the running sum (oh + ol): the
-// lazy accumulation's lo part rounds at ~2^-24 of itself, which over millions of terms
-// (1.4M baselines per pixel) grows to ~5e-9 of the result; folding every 256 terms keeps
+// tile sums' lo part rounds at ~2^-24 of itself, which over millions of terms
+// (1.4M baselines per pixel) grows to ~5e-9 of the result; folding every tile keeps
 // that growth to one tile.
 __device__ __forceinline__ void df_fold(float &oh, float &ol, float ih, float il) {
     float s, e;
@@ -227,10 +115,6 @@ __device__ __forceinline__ int next_item(int *counter, int &s_next) {
     return s_next;
 }
 
-__device__ __forceinline__ void load_tab(float4 *sT, const float4 *__restrict__ gT) {
-    for (int i = threadIdx.x; i < kTabN; i += blockDim.x) sT[i] = gT[i];
-}
-
 // The pointers of one job of a direct launch: a plan's chunk-ordered buffers. A launch
 // serves one job (BATCH false: the kernel parameter J0) or several (BATCH true: work item
 // it belongs to job item_job[it] of the device table jobs, so the sums of several plans
@@ -244,172 +128,468 @@ __device__ __forceinline__ DirectJob job_of(const DirectJob &J0, const DirectJob
         return J0;
 }
 
-// ------------------------------------------------------------- sky -> vis
+// ------------------------------------------------------------- tiles of pairs
 
-// FP32: owner = baselines, streamed = pixels (c real, chunk order).
-template <int VPT, bool BATCH>
-__global__ void __launch_bounds__(kThreads) direct_s2v_f32(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter,
-    const DirectJob J0, const DirectJob *__restrict__ jobs, const int *__restrict__ item_job) {
-    __shared__ float4 sh[kThreads];
-    __shared__ float4 sl[kThreads];
-    __shared__ int s_next;
-    for (int it = blockIdx.x; it < n_items; it = next_item(counter, s_next)) {
-        const WorkItem w = items[it];
-        const DirectJob J = job_of<BATCH>(J0, jobs, item_job, it);
-        const float4 *__restrict__ vh = J.own_hi, *__restrict__ vl = J.own_lo;
-        const float4 *__restrict__ rh_g = J.str_hi, *__restrict__ rl_g = J.str_lo;
-        const float *__restrict__ c = static_cast<const float *>(J.val);
-        float2 *__restrict__ acc = static_cast<float2 *>(J.acc);
-        const float sgn = J.sgn;
-        float3 ph[VPT], pl[VPT];
-        float are[VPT], aim[VPT], cre[VPT], cim[VPT];
+// One work item: 256 owner points [o0, o1) times streamed points [s0, s1). A CTA has 16 consumer
+// warps, 2 producer warps and one issuing warp, and runs as a pipeline on mbarriers:
+//  * producers write the digits and values of the streamed points, 128 at a time,
+//    into one of two tile buffers;
+//  * the tensor cores form the digit products of a chunk of kN streamed points (columns) with
+//    each block of 128 owners (rows; their digits lie in shared memory for the whole item)
+//    into one of two accumulator sets in tensor memory;
+//  * one thread issues those products, as soon as a tile is staged and a set has been read;
+//  * two groups of four warps share a row block, a thread a row: each reads its half of a
+//    chunk's columns into registers and sums them.
+constexpr int kRows = 256;              // owners per work item
+constexpr int kStream = 128;            // streamed points per tile
+constexpr int kConsumers = 2 * kRows;   // threads
+constexpr int kProducers = 64;          // threads, each staging kStream / kProducers points of a tile
+constexpr int kIssuer = kConsumers + kProducers;  // first thread of the issuing warp
+constexpr int kDirectThreads = kIssuer + 32;      // 608: 96 registers a thread
+
+template <class K> struct __align__(128) DirectShared {
+    uint4 own[2][K::Form::kMma * 2][128];      // [row block][mma, K half][row]
+    uint4 dig[2][K::Form::kMma * 2][kStream];  // [buffer][mma, K half][point]
+    typename K::Val val[2][kStream];
+    float red[2][kStream / 32];                // per producer warp: sum of the values' magnitudes
+    typename K::Extra extra;
+    uint64_t done[2][2];                       // [row block][set]: a chunk's products have finished
+    uint64_t read[2][2];                       // [row block][set]: its eight warps have read the set
+    uint64_t staged[2], freed[2];              // [buffer]: tile written / tile summed by every consumer
+    uint32_t tmem;
+    int next, abort;
+};
+
+// Chunks and tiles so far in this CTA (the same in every thread): the n-th use of one of two
+// buffers is buffer n & 1 and barrier phase n >> 1.
+struct DirectPipe {
+    uint32_t tmem, chunks, tiles;
+};
+
+template <class K> __device__ __forceinline__ void pipe_wait(DirectShared<K> &sh, uint64_t *bar, uint32_t parity, int *err) {
+    if (*(volatile int *)&sh.abort || tc::mbar_wait(bar, parity & 1u)) return;
+    *(volatile int *)&sh.abort = 1;  // later waits are skipped and the CTA ends after this item
+    if (err) atomicOr(err, kDevErrStall);
+}
+
+// One producer thread: its points of the tile at s0 (the staged values' magnitudes are summed per
+// warp and pass).
+template <class K, int DIR>
+__device__ __forceinline__ void stage_tile(const DirectJob &J, const WorkItem &w, int s0, DirectShared<K> &sh, int buf) {
+    using Side = std::conditional_t<DIR == 0, typename K::Form::R, typename K::Form::P>;
+    constexpr int kPasses = kStream / kProducers;
+    float4 h[kPasses], l[kPasses];
+    typename K::Val val[kPasses];
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int k = w.o0 + threadIdx.x + v * kThreads;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            if (k < w.o1) {
-                a = vh[k];
-                b = vl[k];
-            }
-            ph[v] = make_float3(a.x, a.y, a.z);
-            pl[v] = make_float3(b.x, b.y, b.z);
-            are[v] = aim[v] = cre[v] = cim[v] = 0.f;
+    for (int p = 0; p < kPasses; ++p) {  // every load in flight before the first is used
+        const int n = s0 + (int)threadIdx.x - kConsumers + p * kProducers;
+        h[p] = l[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        val[p] = typename K::Val{};
+        if (n < w.s1) {
+            h[p] = J.str_hi[n];
+            l[p] = J.str_lo[n];
+            val[p] = K::load(J, n);
         }
-        for (int s0 = w.s0; s0 < w.s1; s0 += kThreads) {
-            __syncthreads();
-            int n = s0 + threadIdx.x;
-            if (n < w.s1) {
-                float4 a = rh_g[n];
-                a.w = c[n];
-                sh[threadIdx.x] = a;
-                sl[threadIdx.x] = rl_g[n];
-            } else {
-                sh[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                sl[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            __syncthreads();
-            const int cnt = min(kThreads, w.s1 - s0);
-            float tre[VPT], tim[VPT];
+    }
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) tre[v] = tim[v] = 0.f;
-#pragma unroll 4
-            for (int q = 0; q < cnt; ++q) {
-                const float4 rh = sh[q], rl = sl[q];
+    for (int p = 0; p < kPasses; ++p) {
+        const int i = (int)threadIdx.x - kConsumers + p * kProducers;
+        tc::write_point<typename K::Form, kStream>(sh.dig[buf], i,
+                                                   tc::point_digits<Side>(h[p], l[p], DIR == 0 ? J.pix_scale : J.vis_scale));
+        sh.val[buf][i] = val[p];
+        if constexpr (K::kMagnitudes) {
+            float mag = K::magnitude(val[p]);
 #pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    float f = phase_f32(ph[v], pl[v], rh, rl);
-                    float sn, cs;
-                    __sincosf(6.28318530717958648f * f, &sn, &cs);
-                    tre[v] = __fmaf_rn(rh.w, cs, tre[v]);
-                    tim[v] = __fmaf_rn(rh.w, sn, tim[v]);
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                kahan_add(are[v], cre[v], tre[v]);
-                kahan_add(aim[v], cim[v], tim[v]);
-            }
+            for (int o = 16; o > 0; o >>= 1) mag += __shfl_xor_sync(0xffffffffu, mag, o);
+            if ((i & 31) == 0) sh.red[buf][i >> 5] = mag;
         }
+    }
+    tc::fence_smem();
+}
+
+// Accumulator columns of a set (tensor memory address without lanes).
+template <class K> __device__ __forceinline__ uint32_t set_columns(int block, uint32_t set) {
+    return ((uint32_t)block * 2u + set) * (K::Form::kAcc * K::kN);
+}
+
+// The issuing thread: the products of every chunk of an item, in order, as tiles are staged and
+// accumulator sets read.
+template <class K>
+__device__ __forceinline__ void issue_chunks(DirectShared<K> &sh, const DirectPipe &pipe, uint32_t chunks, int *err) {
+    constexpr uint32_t kPerTile = kStream / K::kN;
+    const uint64_t own0 = tc::operand_desc(tc::smem_addr(sh.own), sizeof(sh.own[0][0]));
+    const uint64_t dig0 = tc::operand_desc(tc::smem_addr(sh.dig), sizeof(sh.dig[0][0]));
+    for (uint32_t c = 0; c < chunks; ++c) {
+        const uint32_t n = pipe.chunks + c, set = n & 1u, tile = pipe.tiles + c / kPerTile;
+        if (c % kPerTile == 0) pipe_wait(sh, &sh.staged[tile & 1u], tile >> 1, err);
+        const uint64_t dig = dig0 + (((tile & 1u) * sizeof(sh.dig[0]) + (c % kPerTile) * K::kN * 16) >> 4);
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int k = w.o0 + threadIdx.x + v * kThreads;
-            if (k < w.o1) {
-                atomicAdd(&acc[k].x, __fsub_rn(are[v], cre[v]));
-                atomicAdd(&acc[k].y, sgn * __fsub_rn(aim[v], cim[v]));
-            }
+        for (int block = 0; block < 2; ++block) {
+            pipe_wait(sh, &sh.read[block][set], (n >> 1) ^ 1u, err);
+            tc::fence_after();
+            const uint32_t d = pipe.tmem + set_columns<K>(block, set);
+#pragma unroll
+            for (int m = 0; m < K::Form::kMma; ++m)
+                tc::mma<K::kN>(d + K::Form::acc(m) * K::kN, own0 + ((block * sizeof(sh.own[0]) + 2 * m * sizeof(sh.own[0][0])) >> 4),
+                               dig + ((2 * m * sizeof(sh.dig[0][0])) >> 4),
+                               m > 0 && K::Form::acc(m) == K::Form::acc(m - 1));
+            tc::mma_commit(&sh.done[block][set]);
         }
     }
 }
 
-// Double-float: c given in FP64, accumulation returned in FP64.
-template <int VPT, bool BATCH>
-__global__ void __launch_bounds__(kThreads, BATCH && VPT == 2 ? 4 : 0) direct_s2v_df(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter,
-    const DirectJob J0, const DirectJob *__restrict__ jobs, const int *__restrict__ item_job, const float4 *__restrict__ gT) {
-    __shared__ float4 sh[kThreads];
-    __shared__ float4 sl[kThreads];
-    __shared__ float2 sc[kThreads];
-    __shared__ float4 sT[kTabN];
-    __shared__ float red[kThreads / 32];
-    load_tab(sT, gT);
-    __shared__ int s_next;
-    for (int it = blockIdx.x; it < n_items; it = next_item(counter, s_next)) {
-        const WorkItem w = items[it];
-        const DirectJob J = job_of<BATCH>(J0, jobs, item_job, it);
-        const float4 *__restrict__ vh = J.own_hi, *__restrict__ vl = J.own_lo;
-        const float4 *__restrict__ rh_g = J.str_hi, *__restrict__ rl_g = J.str_lo;
-        const double *__restrict__ c = static_cast<const double *>(J.val);
-        double2 *__restrict__ acc = static_cast<double2 *>(J.acc);
-        const float sgn = J.sgn;
-        float3 ph[VPT], pl[VPT];
-        float arh[VPT], arl[VPT], aih[VPT], ail[VPT];  // tile sums, offset by M
-        float orh[VPT], orl[VPT], oih[VPT], oil[VPT];  // running sums, folded per tile
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int k = w.o0 + threadIdx.x + v * kThreads;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-            if (k < w.o1) {
-                a = vh[k];
-                b = vl[k];
-            }
-            ph[v] = make_float3(a.x, a.y, a.z);
-            pl[v] = make_float3(b.x, b.y, b.z);
-            arh[v] = arl[v] = aih[v] = ail[v] = 0.f;
-            orh[v] = orl[v] = oih[v] = oil[v] = 0.f;
+template <class K, int DIR>
+__device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &w, DirectShared<K> &sh, DirectPipe &pipe) {
+    using Form = typename K::Form;
+    using Side = std::conditional_t<DIR == 0, typename Form::P, typename Form::R>;
+    constexpr uint32_t kPerTile = kStream / K::kN;
+    constexpr int kHalf = K::kN / 2, kPart = 8, kParts = kHalf / kPart;  // columns of a chunk per group, per read
+    static_assert(kParts % 2 == 0, "parts alternate between two register sets");
+    const int tid = threadIdx.x;
+    const uint32_t tiles = (uint32_t)(w.s1 - w.s0 + kStream - 1) / kStream;
+    const uint32_t chunks = (uint32_t)(w.s1 - w.s0 + K::kN - 1) / K::kN;
+    if (tid >= kIssuer) {
+        __syncthreads();  // the owners' digits
+        if (tid == kIssuer) issue_chunks(sh, pipe, chunks, J.err);
+        __syncwarp();
+    } else if (tid >= kConsumers) {
+        __syncthreads();
+        for (uint32_t t = 0; t < tiles; ++t) {
+            const uint32_t n = pipe.tiles + t;
+            pipe_wait(sh, &sh.freed[n & 1u], (n >> 1) ^ 1u, J.err);
+            stage_tile<K, DIR>(J, w, w.s0 + (int)t * kStream, sh, n & 1u);
+            __syncwarp();
+            if ((tid & 31) == 0) tc::mbar_arrive(&sh.staged[n & 1u]);
         }
-        for (int s0 = w.s0; s0 < w.s1; s0 += kThreads) {
-            __syncthreads();
-            int n = s0 + threadIdx.x;
-            float mag = 0.f;
-            if (n < w.s1) {
-                sh[threadIdx.x] = rh_g[n];
-                sl[threadIdx.x] = rl_g[n];
-                double cv = c[n];
-                float chi = (float)cv;
-                sc[threadIdx.x] = make_float2(chi, (float)(cv - (double)chi));
-                mag = fabsf(chi);
-            } else {
-                sh[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                sl[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                sc[threadIdx.x] = make_float2(0.f, 0.f);
+    } else {
+        const int block = tid >> 8, half = (tid >> 7) & 1, row = block * 128 + (tid & 127);
+        if (half == 0) {
+            float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
+            if (w.o0 + row < w.o1) {
+                h = J.own_hi[w.o0 + row];
+                l = J.own_lo[w.o0 + row];
             }
-            // |c (cos, sin)| <= |c| (1 + 2^-23): S = 1.01 sum |c| bounds each partial sum
-            const float M = tile_offset(1.01f * block_sum(mag, red));
-            const int cnt = min(kThreads, w.s1 - s0);
+            tc::write_point<Form, 128>(sh.own[block], tid & 127,
+                                       tc::point_digits<Side>(h, l, DIR == 0 ? J.vis_scale : J.pix_scale));
+            tc::fence_smem();
+        }
+        __syncthreads();
+        const uint32_t lanes = pipe.tmem + ((uint32_t)(tid & 96) << 16) + half * kHalf;  // this warp's 32 lanes
+        typename K::Sum sum;
+        sum.clear();
+        // A part (8 columns of every accumulator) is read while the part before it is summed.
+        float d[2][Form::kAcc][kPart];
+        auto read_part = [&](uint32_t set, int p) {
 #pragma unroll
-            for (int v = 0; v < VPT; ++v) arh[v] = aih[v] = M;
-#pragma unroll 4
-            for (int q = 0; q < cnt; ++q) {
-                const float4 rh = sh[q], rl = sl[q];
-                const float2 cv = sc[q];
+            for (int a = 0; a < Form::kAcc; ++a)
+                tc::tmem_load8(d[p & 1][a], lanes + set_columns<K>(block, set) + a * K::kN + p * kPart);
+        };
+        auto open_chunk = [&](uint32_t c) {  // the chunk's products are done: read its first part
+            const uint32_t n = pipe.chunks + c;
+            pipe_wait(sh, &sh.done[block][n & 1u], n >> 1, J.err);
+            __syncwarp();
+            tc::fence_after();
+            read_part(n & 1u, 0);
+        };
+        open_chunk(0);
+        for (uint32_t c = 0; c < chunks; ++c) {
+            const uint32_t set = (pipe.chunks + c) & 1u, tile = pipe.tiles + c / kPerTile, buf = tile & 1u;
+            if (c % kPerTile == 0) {
+                pipe_wait(sh, &sh.staged[buf], tile >> 1, J.err);
+                sum.begin(sh.red[buf]);
+            }
+            const auto *val = &sh.val[buf][(c % kPerTile) * K::kN + half * kHalf];
 #pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    float fh, fl, reh, rel, imh, iml;
-                    phase_df(ph[v], pl[v], rh, rl, fh, fl);
-                    cis_tab(fh, fl, sT, reh, rel, imh, iml);
-                    float th, tl;
-                    df_mul(cv.x, cv.y, reh, rel, th, tl);
-                    df_acc_off(arh[v], arl[v], th, tl);
-                    df_mul(cv.x, cv.y, imh, iml, th, tl);
-                    df_acc_off(aih[v], ail[v], th, tl);
+            for (int p = 0; p < kParts; ++p) {
+#pragma unroll
+                for (int a = 0; a < Form::kAcc; ++a) tc::tmem_load_wait(d[p & 1][a]);
+                if (p + 1 < kParts) {
+                    read_part(set, p + 1);
+                } else {
+                    tc::fence_before();
+                    __syncwarp();
+                    if ((tid & 31) == 0) tc::mbar_arrive(&sh.read[block][set]);
+                    if (c + 1 < chunks) open_chunk(c + 1);
                 }
+                sum.chunk(d[p & 1], val + p * kPart, p * kPart, sh.extra);
             }
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                df_fold(orh[v], orl[v], __fsub_rn(arh[v], M), arl[v]);
-                df_fold(oih[v], oil[v], __fsub_rn(aih[v], M), ail[v]);
-                arl[v] = ail[v] = 0.f;
+            if (c % kPerTile == kPerTile - 1 || c + 1 == chunks) {
+                sum.end();
+                __syncwarp();
+                if ((tid & 31) == 0) tc::mbar_arrive(&sh.freed[buf]);
             }
         }
+        if (*(volatile int *)&sh.abort) sum.poison();
+        if (w.o0 + row < w.o1) sum.store(J, w.o0 + row);
+    }
+    pipe.chunks += chunks;
+    pipe.tiles += tiles;
+}
+
+template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShared<K> &sh) {
+    static_assert(4 * K::Form::kAcc * K::kN <= 512 && K::kN % 16 == 0 && kStream % K::kN == 0, "tensor memory of an SM");
+    if (threadIdx.x < 32) tc::tmem_alloc(&sh.tmem, 512);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) {
+            for (int b = 0; b < 2; ++b) {
+                tc::mbar_init(&sh.done[b][i], 1);
+                tc::mbar_init(&sh.read[b][i], 8);
+            }
+            tc::mbar_init(&sh.staged[i], kProducers / 32);
+            tc::mbar_init(&sh.freed[i], kConsumers / 32);
+        }
+        sh.abort = 0;
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    return {sh.tmem, 0u, 0u};
+}
+
+template <class K> __device__ __forceinline__ void direct_end(DirectShared<K> &sh, const DirectPipe &pipe) {
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    if (threadIdx.x < 32) tc::tmem_free(pipe.tmem, 512);
+}
+
+// ------------------------------------------------------------- FP32
+
+// exp(j 2 pi f) for f = A 2^-14 + B 2^-25 turns (A whole, |A| < 2^24): the whole turns of A go
+// exactly; the rest (|f| <~ 0.6) is rounded once, in radians. sin.approx and cos.approx multiply
+// by fl(1 / 2 pi) = (1 - 4.0e-8) / 2 pi and truncate; with 2 pi rounded to float, (1 + 2.8e-8) 2 pi,
+// every phase comes out short and the mean of the cosine over a turn is off by 1.8e-8, and a
+// sum of 1.5M positive values (a long baseline's visibility) by that times its total. One
+// column in six (j: the column) takes the next float above 2 pi instead, (1 + 1.04e-7) 2 pi, so that
+// the factor is 1 + 4.05e-8 on average and the mean error of the cosine vanishes.
+__device__ __forceinline__ void cis_f32(float A, float B, int j, float &cs, float &sn) {
+    const float k = j % 6 == 5 ? 6.28318595886230469f : 6.28318548202514648f;
+    const float n = tc::nearest(A, 0x1p-14f);
+    const float a = __fmaf_rn(n, -0x1p14f, A);
+    const float x = __fmaf_rn(a, k * 0x1p-14f, __fmul_rn(B, k * 0x1p-25f));
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(sn) : "f"(x));
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(cs) : "f"(x));
+}
+
+struct NoExtra {};
+
+template <int DIR> struct F32Sum;
+template <> struct F32Sum<0> {
+    float re, im, cre, cim, tre, tim;
+    __device__ __forceinline__ void clear() { re = im = cre = cim = 0.f; }
+    __device__ __forceinline__ void poison() { re = im = __int_as_float(0x7fc00000); }
+    __device__ __forceinline__ void begin(const float *) { tre = tim = 0.f; }
+    template <int N>
+    __device__ __forceinline__ void chunk(const float (&d)[2][N], const float *c, int j0, const NoExtra &) {
 #pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int k = w.o0 + threadIdx.x + v * kThreads;
-            if (k < w.o1) {
-                atomicAdd(&acc[k].x, (double)orh[v] + (double)orl[v]);
-                atomicAdd(&acc[k].y, (double)sgn * ((double)oih[v] + (double)oil[v]));
+        for (int j = 0; j < N; j += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(c + j);
+            const float cv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float cs, sn;
+                cis_f32(d[0][j + i], d[1][j + i], j0 + j + i, cs, sn);
+                tre = __fmaf_rn(cv[i], cs, tre);
+                tim = __fmaf_rn(cv[i], sn, tim);
             }
         }
     }
+    __device__ __forceinline__ void end() {
+        kahan_add(re, cre, tre);
+        kahan_add(im, cim, tim);
+    }
+    __device__ __forceinline__ void store(const DirectJob &J, int k) const {
+        float2 *acc = static_cast<float2 *>(J.acc);
+        atomicAdd(&acc[k].x, __fsub_rn(re, cre));
+        atomicAdd(&acc[k].y, J.sgn * __fsub_rn(im, cim));
+    }
+};
+template <> struct F32Sum<1> {
+    float re, cre, tre;
+    __device__ __forceinline__ void clear() { re = cre = 0.f; }
+    __device__ __forceinline__ void poison() { re = __int_as_float(0x7fc00000); }
+    __device__ __forceinline__ void begin(const float *) { tre = 0.f; }
+    template <int N>
+    __device__ __forceinline__ void chunk(const float (&d)[2][N], const float2 *V, int j0, const NoExtra &) {
+#pragma unroll
+        for (int j = 0; j < N; j += 2) {
+            const float4 v = *reinterpret_cast<const float4 *>(V + j);
+            const float vr[2] = {v.x, v.z}, vi[2] = {v.y, v.w};
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                float cs, sn;
+                cis_f32(d[0][j + i], d[1][j + i], j0 + j + i, cs, sn);
+                // Re(V e^{-isign j 2 pi t}) = Vr cos + isign Vi sin
+                tre = __fmaf_rn(vr[i], cs, __fmaf_rn(vi[i], sn, tre));
+            }
+        }
+    }
+    __device__ __forceinline__ void end() { kahan_add(re, cre, tre); }
+    __device__ __forceinline__ void store(const DirectJob &J, int k) const {
+        atomicAdd(static_cast<float *>(J.acc) + k, __fsub_rn(re, cre));
+    }
+};
+
+template <int DIR> struct F32Kind {
+    using Form = tc::F32Form;
+    using Val = std::conditional_t<DIR == 0, float, float2>;
+    using Sum = F32Sum<DIR>;
+    using Extra = NoExtra;
+    static constexpr int kN = 64;
+    static constexpr bool kMagnitudes = false;
+    static __device__ __forceinline__ Val load(const DirectJob &J, int n) {
+        if constexpr (DIR == 0) {
+            return static_cast<const float *>(J.val)[n];
+        } else {
+            float2 v = static_cast<const float2 *>(J.val)[n];
+            v.y *= J.sgn;
+            return v;
+        }
+    }
+};
+
+// ------------------------------------------------------------- double-float
+
+constexpr int kDfTab = 1024;   // entries per turn of the sine table
+constexpr int kDfCopies = 8;   // one copy of each entry per lane of a quarter warp
+
+struct DfTable {
+    float4 e[kDfTab * kDfCopies];  // entry m, copy c: (cos_h, cos_l, sin_h, sin_l) of 2 pi m / 1024
+};
+
+// exp(j 2 pi f) as (reh + rel) + j (imh + iml), f = (A - 1.5 2^23) / 1024 + B 2^-20 + C1 2^-31 + C2 2^-42
+// turns (A whole). The nearest 1/1024 turn to the rest joins A and picks the table entry (the
+// table's hi parts, exact floats); the remainder x (in units of 2^-20 turn, |x| <= 2^9) is formed
+// exactly but for its last rounding (2^-36 turn) and rotates the entry through cos x - 1 =
+// -x^2/2, sin x = x - x^3/6 in plain float. tab: the shared address of this lane's copy of the table.
+__device__ __forceinline__ void cis_df(float A, float B, float C1, float C2, uint32_t tab, float &reh, float &rel,
+                                       float &imh, float &iml) {
+    const float tt = __fmaf_rn(__fmaf_rn(C1, 0x1p-11f, B), 0x1p-10f, A);  // 1.5 2^23 + entry
+    const float d = __fmaf_rn(__fsub_rn(tt, A), -1024.f, B);
+    const float x = __fmaf_rn(C2, 0x1p-22f, __fmaf_rn(C1, 0x1p-11f, d));
+    const uint32_t at = ((__float_as_uint(tt) & (kDfTab - 1)) * (16u * kDfCopies)) + tab;
+    float4 tb;
+    asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(tb.x), "=f"(tb.y), "=f"(tb.z), "=f"(tb.w) : "r"(at));
+    constexpr float k = 6.28318530717958648f * 0x1p-20f;
+    const float x2 = __fmul_rn(x, x);
+    const float cm = __fmul_rn(x2, -0.5f * k * k);
+    const float sx = __fmul_rn(x, __fmaf_rn(x2, -k * k * k / 6.0f, k));
+    reh = tb.x;
+    rel = __fmaf_rn(-tb.z, sx, __fmaf_rn(tb.x, cm, tb.y));
+    imh = tb.z;
+    iml = __fmaf_rn(tb.x, sx, __fmaf_rn(tb.z, cm, tb.w));
 }
+
+// Offset double-float accumulation of one streamed tile: h += (ch + cl)(eh + el). The running
+// high sum starts at a power of two M above twice the tile's sum of term magnitudes S, so
+// it stays in [M - S, M + S]: h - h' is exact, and the part of both products that the two
+// FMAs rounded off is recovered by FMAs on that difference and collected in l with cl eh.
+// At the tile's end h - M is exact (Sterbenz).
+struct DfAcc {
+    float h, l, oh, ol;  // tile sum (offset by M) and running sum
+    __device__ __forceinline__ void mac(float ch, float cl, float eh, float el) {
+        const float s = __fmaf_rn(ch, el, __fmaf_rn(ch, eh, h));
+        float u = __fmaf_rn(ch, eh, __fsub_rn(h, s));
+        u = __fmaf_rn(cl, eh, __fmaf_rn(ch, el, u));
+        h = s;
+        l = __fadd_rn(l, u);
+    }
+};
+
+template <int DIR, class T> struct DfSum {
+    static constexpr int kV = DIR == 0 ? 2 : 1;  // re and im, or one real sum
+    DfAcc a[kV];
+    float M;
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int c = 0; c < kV; ++c) a[c].oh = a[c].ol = 0.f;
+    }
+    __device__ __forceinline__ void poison() { a[0].oh = a[kV - 1].oh = __int_as_float(0x7fc00000); }
+    __device__ __forceinline__ void begin(const float *red) {
+        float S = 0.f;
+#pragma unroll
+        for (int i = 0; i < kStream / 32; ++i) S += red[i];
+        M = tile_offset(1.01f * S);
+#pragma unroll
+        for (int c = 0; c < kV; ++c) {
+            a[c].h = M;
+            a[c].l = 0.f;
+        }
+    }
+    template <int N, class Val>
+    __device__ __forceinline__ void chunk(const float (&d)[4][N], const Val *v, int, const DfTable &table) {
+        const uint32_t tab = tc::smem_addr(&table.e[threadIdx.x & (kDfCopies - 1)]);
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            float reh, rel, imh, iml;
+            cis_df(d[0][j], d[1][j], d[2][j], d[3][j], tab, reh, rel, imh, iml);
+            if constexpr (DIR == 0) {
+                const float2 c = v[j];
+                a[0].mac(c.x, c.y, reh, rel);
+                a[kV - 1].mac(c.x, c.y, imh, iml);
+            } else {
+                const float4 c = v[j];
+                a[0].mac(c.x, c.y, reh, rel);
+                a[0].mac(c.z, c.w, imh, iml);
+            }
+        }
+    }
+    __device__ __forceinline__ void end() {
+#pragma unroll
+        for (int c = 0; c < kV; ++c) df_fold(a[c].oh, a[c].ol, __fsub_rn(a[c].h, M), a[c].l);
+    }
+    __device__ __forceinline__ void store(const DirectJob &J, int k) const {
+        T *acc = static_cast<T *>(J.acc) + (size_t)k * kV;
+        atomicAdd(acc, (T)((double)a[0].oh + (double)a[0].ol));
+        if constexpr (DIR == 0) atomicAdd(acc + 1, (T)((double)J.sgn * ((double)a[1].oh + (double)a[1].ol)));
+    }
+};
+
+// The sine table takes 128 KB: 8 copies make every read of a quarter warp conflict-free, where
+// 8 lanes reading one table at random met ~2.6 times in a bank group.
+// T: the plan's real type (float: the wide path).
+template <int DIR, class T> struct DfKind {
+    using Form = tc::DfForm;
+    using Val = std::conditional_t<DIR == 0, float2, float4>;
+    using Sum = DfSum<DIR, T>;
+    using Extra = DfTable;
+    static constexpr int kN = 32;
+    static constexpr bool kMagnitudes = true;
+    // (c_h, c_l), or (Vr_h, Vr_l, Vi_h, Vi_l) with isign on Vi
+    static __device__ __forceinline__ Val load(const DirectJob &J, int n) {
+        const T *v = static_cast<const T *>(J.val) + (size_t)n * (DIR == 0 ? 1 : 2);
+        const float rh = (float)v[0], rl = (float)(v[0] - (T)rh);
+        if constexpr (DIR == 0) {
+            return make_float2(rh, rl);
+        } else {
+            const T vi = (T)J.sgn * v[1];
+            const float ih = (float)vi;
+            return make_float4(rh, rl, ih, (float)(vi - (T)ih));
+        }
+    }
+    // each pair adds at most |c| or |Vr| + |Vi| to a sum
+    static __device__ __forceinline__ float magnitude(const Val &v) {
+        if constexpr (DIR == 0) return fabsf(v.x);
+        else return fabsf(v.x) + fabsf(v.z);
+    }
+};
+
+// gT (double-float): exp(j 2 pi m / 2048), m = 0 .. 2047, as float pairs; every other entry is kept.
+template <class K, int DIR, bool BATCH>
+__global__ void __launch_bounds__(kDirectThreads, 1)
+    direct_kernel(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter, const DirectJob J0,
+                  const DirectJob *__restrict__ jobs, const int *__restrict__ item_job, const float4 *__restrict__ gT) {
+    extern __shared__ __align__(128) unsigned char direct_smem[];
+    DirectShared<K> &sh = *reinterpret_cast<DirectShared<K> *>(direct_smem);
+    DirectPipe pipe = direct_begin(sh);
+    if constexpr (K::kMagnitudes)
+        for (int i = threadIdx.x; i < kDfTab * kDfCopies; i += kDirectThreads) sh.extra.e[i] = gT[2 * (i / kDfCopies)];
+    for (int it = blockIdx.x; it < n_items && !sh.abort; it = next_item(counter, sh.next))
+        direct_item<K, DIR>(job_of<BATCH>(J0, jobs, item_job, it), items[it], sh, pipe);
+    direct_end(sh, pipe);
+}
+
+// ------------------------------------------------------------- FP64
 
 // Plain FP64 reference form.
 template <int VPT>
@@ -461,166 +641,6 @@ __global__ void __launch_bounds__(kThreads) direct_s2v_f64(const WorkItem *__res
                 atomicAdd(&acc[k].x, are[v]);
                 atomicAdd(&acc[k].y, sgn * aim[v]);
             }
-        }
-    }
-}
-
-// ------------------------------------------------------------- vis -> sky
-
-// FP32: owner = pixels, streamed = baselines (V complex, chunk order). Output real.
-template <int VPT, bool BATCH>
-__global__ void __launch_bounds__(kThreads) direct_v2s_f32(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter,
-    const DirectJob J0, const DirectJob *__restrict__ jobs, const int *__restrict__ item_job) {
-    __shared__ float4 sh[kThreads];
-    __shared__ float4 sl[kThreads];
-    __shared__ int s_next;
-    for (int it = blockIdx.x; it < n_items; it = next_item(counter, s_next)) {
-        const WorkItem w = items[it];
-        const DirectJob J = job_of<BATCH>(J0, jobs, item_job, it);
-        const float4 *__restrict__ rh_g = J.own_hi, *__restrict__ rl_g = J.own_lo;
-        const float4 *__restrict__ vh = J.str_hi, *__restrict__ vl = J.str_lo;
-        const float2 *__restrict__ V = static_cast<const float2 *>(J.val);
-        float *__restrict__ acc = static_cast<float *>(J.acc);
-        const float sgn = J.sgn;
-        float3 rh[VPT], rl[VPT];
-        float a[VPT], ca[VPT];
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int n = w.o0 + threadIdx.x + v * kThreads;
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-            if (n < w.o1) {
-                x = rh_g[n];
-                y = rl_g[n];
-            }
-            rh[v] = make_float3(x.x, x.y, x.z);
-            rl[v] = make_float3(y.x, y.y, y.z);
-            a[v] = ca[v] = 0.f;
-        }
-        for (int s0 = w.s0; s0 < w.s1; s0 += kThreads) {
-            __syncthreads();
-            int k = s0 + threadIdx.x;
-            if (k < w.s1) {
-                float4 p = vh[k], q = vl[k];
-                float2 val = V[k];
-                p.w = val.x;
-                q.w = sgn * val.y;
-                sh[threadIdx.x] = p;
-                sl[threadIdx.x] = q;
-            } else {
-                sh[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                sl[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            __syncthreads();
-            const int cnt = min(kThreads, w.s1 - s0);
-            float ta[VPT];
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) ta[v] = 0.f;
-#pragma unroll 4
-            for (int q = 0; q < cnt; ++q) {
-                const float4 ph4 = sh[q], pl4 = sl[q];
-                const float3 ph = make_float3(ph4.x, ph4.y, ph4.z), pl = make_float3(pl4.x, pl4.y, pl4.z);
-#pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    float4 r4h = make_float4(rh[v].x, rh[v].y, rh[v].z, 0.f);
-                    float4 r4l = make_float4(rl[v].x, rl[v].y, rl[v].z, 0.f);
-                    float f = phase_f32(ph, pl, r4h, r4l);
-                    float sn, cs;
-                    __sincosf(6.28318530717958648f * f, &sn, &cs);
-                    // Re(V e^{-isign j 2 pi t}) = Vr cos + isign Vi sin
-                    ta[v] = __fmaf_rn(ph4.w, cs, __fmaf_rn(pl4.w, sn, ta[v]));
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) kahan_add(a[v], ca[v], ta[v]);
-        }
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int n = w.o0 + threadIdx.x + v * kThreads;
-            if (n < w.o1) atomicAdd(&acc[n], __fsub_rn(a[v], ca[v]));
-        }
-    }
-}
-
-template <int VPT, bool BATCH>
-__global__ void __launch_bounds__(kThreads) direct_v2s_df(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter,
-    const DirectJob J0, const DirectJob *__restrict__ jobs, const int *__restrict__ item_job, const float4 *__restrict__ gT) {
-    __shared__ float4 sh[kThreads];
-    __shared__ float4 sl[kThreads];
-    __shared__ float4 sv[kThreads];
-    __shared__ float4 sT[kTabN];
-    __shared__ float red[kThreads / 32];
-    load_tab(sT, gT);
-    __shared__ int s_next;
-    for (int it = blockIdx.x; it < n_items; it = next_item(counter, s_next)) {
-        const WorkItem w = items[it];
-        const DirectJob J = job_of<BATCH>(J0, jobs, item_job, it);
-        const float4 *__restrict__ rh_g = J.own_hi, *__restrict__ rl_g = J.own_lo;
-        const float4 *__restrict__ vh = J.str_hi, *__restrict__ vl = J.str_lo;
-        const double2 *__restrict__ V = static_cast<const double2 *>(J.val);
-        double *__restrict__ acc = static_cast<double *>(J.acc);
-        const float sgn = J.sgn;
-        float4 rh[VPT], rl[VPT];
-        float ah[VPT], al[VPT], oh[VPT], ol[VPT];  // tile sums (offset by M) and running sums
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int n = w.o0 + threadIdx.x + v * kThreads;
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-            if (n < w.o1) {
-                x = rh_g[n];
-                y = rl_g[n];
-            }
-            rh[v] = x;
-            rl[v] = y;
-            ah[v] = al[v] = oh[v] = ol[v] = 0.f;
-        }
-        for (int s0 = w.s0; s0 < w.s1; s0 += kThreads) {
-            __syncthreads();
-            int k = s0 + threadIdx.x;
-            float mag = 0.f;
-            if (k < w.s1) {
-                sh[threadIdx.x] = vh[k];
-                sl[threadIdx.x] = vl[k];
-                double2 val = V[k];
-                double vi = (double)sgn * val.y;
-                float rh_ = (float)val.x, ih_ = (float)vi;
-                sv[threadIdx.x] = make_float4(rh_, (float)(val.x - (double)rh_), ih_, (float)(vi - (double)ih_));
-                mag = fabsf(rh_) + fabsf(ih_);
-            } else {
-                sh[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                sl[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-                sv[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            // each pair adds Vre cos + Vim sin: S = 1.01 sum (|Vre| + |Vim|) bounds the partial sums
-            const float M = tile_offset(1.01f * block_sum(mag, red));
-            const int cnt = min(kThreads, w.s1 - s0);
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) ah[v] = M;
-#pragma unroll 4
-            for (int q = 0; q < cnt; ++q) {
-                const float4 ph4 = sh[q], pl4 = sl[q], val = sv[q];
-                const float3 ph = make_float3(ph4.x, ph4.y, ph4.z), pl = make_float3(pl4.x, pl4.y, pl4.z);
-#pragma unroll
-                for (int v = 0; v < VPT; ++v) {
-                    float fh, fl, reh, rel, imh, iml;
-                    phase_df(ph, pl, rh[v], rl[v], fh, fl);
-                    cis_tab(fh, fl, sT, reh, rel, imh, iml);
-                    float th, tl;
-                    df_mul(val.x, val.y, reh, rel, th, tl);
-                    df_acc_off(ah[v], al[v], th, tl);
-                    df_mul(val.z, val.w, imh, iml, th, tl);
-                    df_acc_off(ah[v], al[v], th, tl);
-                }
-            }
-#pragma unroll
-            for (int v = 0; v < VPT; ++v) {
-                df_fold(oh[v], ol[v], __fsub_rn(ah[v], M), al[v]);
-                al[v] = 0.f;
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < VPT; ++v) {
-            int n = w.o0 + threadIdx.x + v * kThreads;
-            if (n < w.o1) atomicAdd(&acc[n], (double)oh[v] + (double)ol[v]);
         }
     }
 }
@@ -693,108 +713,99 @@ void launch_gather_weight(const double *w, const int32_t *perm, int64_t n, doubl
     check_cuda(cudaGetLastError(), "gather_weight");
 }
 
-int direct_tile(int vpt) { return kThreads * vpt; }
+int direct_tile(int kind) { return kind == kDirectF64 ? kTile : kRows; }
 
-static unsigned grid_for(int64_t n_items) {
-    static int sms = 0;
-    if (sms == 0) {
+int direct_owners_per_thread(int kind) { return kind == kDirectF64 ? kPerThread : 1; }
+
+static int sm_count() {
+    static std::atomic<int> sms{0};
+    int n = sms.load();
+    if (n == 0) {
         int dev = 0;
         cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 152;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        if (n <= 0) n = 152;
+        sms.store(n);
     }
-    int64_t g = std::min<int64_t>(n_items, (int64_t)sms * 4);
-    return (unsigned)std::max<int64_t>(g, 1);
+    return n;
 }
 
-void launch_direct_s2v_f32(const WorkItem *items, int64_t n, int *counter, const float4 *vh, const float4 *vl, const float4 *rh,
-                           const float4 *rl, const float *c, float2 *acc, int isign, int vpt, cudaStream_t s) {
-    if (n <= 0) return;
-    const DirectJob J{vh, vl, rh, rl, c, acc, (float)isign};
-    if (vpt == 4)
-        direct_s2v_f32<4, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr);
-    else
-        direct_s2v_f32<2, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr);
-    check_cuda(cudaGetLastError(), "direct_s2v_f32");
+// A persistent grid: the CTAs that are resident together (per_sm on every SM), at most one per item.
+static unsigned grid_for(int64_t n_items, int per_sm) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_items, (int64_t)sm_count() * per_sm));
 }
 
-void launch_direct_s2v_df(const WorkItem *items, int64_t n, int *counter, const float4 *vh, const float4 *vl, const float4 *rh,
-                          const float4 *rl, const double *c, double2 *acc, const float4 *tab, int isign,
-                          int vpt, cudaStream_t s) {
-    if (n <= 0) return;
-    const DirectJob J{vh, vl, rh, rl, c, acc, (float)isign};
-    if (vpt == 4)
-        direct_s2v_df<4, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr, tab);
-    else
-        direct_s2v_df<2, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr, tab);
-    check_cuda(cudaGetLastError(), "direct_s2v_df");
+// Dynamic shared memory of a kernel, allowed once per device (Once names the kernel).
+template <class Once, class F> static void allow_smem(F kernel, size_t bytes) {
+    static std::atomic<uint64_t> done[4];
+    int dev = 0;
+    check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+    if (dev < 256 && (done[dev / 64].load() >> (dev % 64) & 1)) return;
+    check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+               "cudaFuncSetAttribute");
+    if (dev < 256) done[dev / 64].fetch_or(uint64_t(1) << (dev % 64));
 }
 
-void launch_direct_s2v_f64(const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv, const double *pxyz,
-                           int64_t np, const double *c, double2 *acc, int isign, int vpt, cudaStream_t s) {
+template <class K, int DIR, bool BATCH> struct DirectOnce {};
+
+template <class K, int DIR, bool BATCH>
+static void launch_one(const WorkItem *items, int64_t n, int *counter, const DirectJob &J, const DirectJob *jobs,
+                       const int *item_job, const float4 *tab, cudaStream_t s) {
+    constexpr size_t smem = sizeof(DirectShared<K>);
+    static_assert(smem <= 226 * 1024, "shared memory of an SM");
+    allow_smem<DirectOnce<K, DIR, BATCH>>(direct_kernel<K, DIR, BATCH>, smem);
+    direct_kernel<K, DIR, BATCH><<<grid_for(n, 1), kDirectThreads, smem, s>>>(items, (int)n, counter, J, jobs,
+                                                                                 item_job, tab);
+    check_cuda(cudaGetLastError(), "direct sums");
+}
+
+template <bool BATCH>
+static void launch_kind(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob &J,
+                        const DirectJob *jobs, const int *item_job, const float4 *tab, cudaStream_t s) {
+#define HVOX_DIRECT(...)                                                                            \
+    if (dir == 0)                                                                                   \
+        launch_one<__VA_ARGS__(0), 0, BATCH>(items, n, counter, J, jobs, item_job, tab, s);         \
+    else                                                                                            \
+        launch_one<__VA_ARGS__(1), 1, BATCH>(items, n, counter, J, jobs, item_job, tab, s)
+#define HVOX_F32(D) F32Kind<D>
+#define HVOX_DF(D) DfKind<D, double>
+#define HVOX_WIDE(D) DfKind<D, float>
+    if (kind == kDirectF32) {
+        HVOX_DIRECT(HVOX_F32);
+    } else if (kind == kDirectDf) {
+        HVOX_DIRECT(HVOX_DF);
+    } else {
+        HVOX_DIRECT(HVOX_WIDE);
+    }
+#undef HVOX_DIRECT
+#undef HVOX_F32
+#undef HVOX_DF
+#undef HVOX_WIDE
+}
+
+void launch_direct(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob &J,
+                   const float4 *tab, cudaStream_t s) {
+    if (n > 0) launch_kind<false>(kind, dir, items, n, counter, J, nullptr, nullptr, tab, s);
+}
+
+void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob *jobs,
+                         const int *item_job, const float4 *tab, cudaStream_t s) {
+    if (n > 0) launch_kind<true>(kind, dir, items, n, counter, DirectJob{}, jobs, item_job, tab, s);
+}
+
+void launch_direct_s2v_f64(const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
+                           const double *pxyz, int64_t np, const double *c, double2 *acc, int isign, cudaStream_t s) {
     if (n <= 0) return;
-    if (vpt == 4)
-        direct_s2v_f64<4><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, vxyz, nv, pxyz, np, c, acc, (double)isign);
-    else
-        direct_s2v_f64<2><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, vxyz, nv, pxyz, np, c, acc, (double)isign);
+    direct_s2v_f64<kPerThread><<<grid_for(n, 4), kThreads, 0, s>>>(items, (int)n, counter, vxyz, nv, pxyz, np, c, acc,
+                                                                   (double)isign);
     check_cuda(cudaGetLastError(), "direct_s2v_f64");
 }
 
-void launch_direct_v2s_f32(const WorkItem *items, int64_t n, int *counter, const float4 *rh, const float4 *rl, const float4 *vh,
-                           const float4 *vl, const float2 *V, float *acc, int isign, int vpt, cudaStream_t s) {
+void launch_direct_v2s_f64(const WorkItem *items, int64_t n, int *counter, const double *pxyz, int64_t np,
+                           const double *vxyz, int64_t nv, const double2 *V, double *acc, int isign, cudaStream_t s) {
     if (n <= 0) return;
-    const DirectJob J{rh, rl, vh, vl, V, acc, (float)isign};
-    if (vpt == 4)
-        direct_v2s_f32<4, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr);
-    else
-        direct_v2s_f32<2, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr);
-    check_cuda(cudaGetLastError(), "direct_v2s_f32");
-}
-
-void launch_direct_v2s_df(const WorkItem *items, int64_t n, int *counter, const float4 *rh, const float4 *rl, const float4 *vh,
-                          const float4 *vl, const double2 *V, double *acc, const float4 *tab, int isign,
-                          int vpt, cudaStream_t s) {
-    if (n <= 0) return;
-    const DirectJob J{rh, rl, vh, vl, V, acc, (float)isign};
-    if (vpt == 4)
-        direct_v2s_df<4, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr, tab);
-    else
-        direct_v2s_df<2, false><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, J, nullptr, nullptr, tab);
-    check_cuda(cudaGetLastError(), "direct_v2s_df");
-}
-
-// Several jobs' work items in one launch (kind 0 FP32, 1 double-float; dir 0 sky -> vis,
-// 1 vis -> sky); jobs and item_job in device memory, items sorted largest first.
-void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob *jobs,
-                         const int *item_job, const float4 *tab, int vpt, cudaStream_t s) {
-    if (n <= 0) return;
-    const DirectJob J0{};
-    const unsigned g = grid_for(n);
-#define HVOX_BATCH(KERNEL, ...)                                                                              \
-    if (vpt == 4)                                                                                            \
-        KERNEL<4, true><<<g, kThreads, 0, s>>>(items, (int)n, counter, J0, jobs, item_job __VA_ARGS__);      \
-    else                                                                                                     \
-        KERNEL<2, true><<<g, kThreads, 0, s>>>(items, (int)n, counter, J0, jobs, item_job __VA_ARGS__);
-    if (kind == 0 && dir == 0) {
-        HVOX_BATCH(direct_s2v_f32)
-    } else if (kind == 0) {
-        HVOX_BATCH(direct_v2s_f32)
-    } else if (dir == 0) {
-        HVOX_BATCH(direct_s2v_df, , tab)
-    } else {
-        HVOX_BATCH(direct_v2s_df, , tab)
-    }
-#undef HVOX_BATCH
-    check_cuda(cudaGetLastError(), "direct_batch");
-}
-
-void launch_direct_v2s_f64(const WorkItem *items, int64_t n, int *counter, const double *pxyz, int64_t np, const double *vxyz,
-                           int64_t nv, const double2 *V, double *acc, int isign, int vpt, cudaStream_t s) {
-    if (n <= 0) return;
-    if (vpt == 4)
-        direct_v2s_f64<4><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, pxyz, np, vxyz, nv, V, acc, (double)isign);
-    else
-        direct_v2s_f64<2><<<grid_for(n), kThreads, 0, s>>>(items, (int)n, counter, pxyz, np, vxyz, nv, V, acc, (double)isign);
+    direct_v2s_f64<kPerThread><<<grid_for(n, 4), kThreads, 0, s>>>(items, (int)n, counter, pxyz, np, vxyz, nv, V, acc,
+                                                                   (double)isign);
     check_cuda(cudaGetLastError(), "direct_v2s_f64");
 }
 
@@ -820,93 +831,70 @@ namespace {
 
 constexpr int64_t kNoAllocMaxPoints = int64_t(1) << 19;  // n_pix + n_vis <= 524,288
 
-// hi and lo float splits of the pixel and baseline coordinates: 2 * 524,288 float4 = 16 MiB.
-__device__ __align__(256) float4 g_noalloc_scratch[2 * kNoAllocMaxPoints];
+// hi and lo float splits of the pixel and baseline coordinates: 2 * 524,288 float4 = 16 MiB; then
+// the largest |coordinate| of the pixels and of the baselines of the call as float bits.
+__device__ __align__(256) float4 g_noalloc_scratch[2 * kNoAllocMaxPoints + 1];
 
-__global__ void noalloc_split_kernel(const double *__restrict__ xyz, int64_t n, float4 *__restrict__ hi,
-                                     float4 *__restrict__ lo) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float h[3], l[3];
-    for (int d = 0; d < 3; ++d) {
-        double x = xyz[3 * i + d];
-        h[d] = (float)x;
-        l[d] = (float)(x - (double)h[d]);
+// One launch before the sums: coordinate splits of pixels and baselines, V cleared, and the
+// largest |coordinate| of each set (non-negative floats order as integers; top[0..1] zero at launch).
+__global__ void noalloc_prepare_kernel(const double *__restrict__ pix, int64_t n_pix, const double *__restrict__ uvw,
+                                       int64_t n_vis, float4 *__restrict__ scratch, unsigned *__restrict__ top,
+                                       float2 *__restrict__ V) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    float m = 0.f;
+    const bool p = i < n_pix;
+    if (i < n_pix + n_vis) {
+        const int64_t k = p ? i : i - n_pix;
+        const double *xyz = (p ? pix : uvw) + 3 * k;
+        float4 *hi = p ? scratch : scratch + 2 * n_pix, *lo = hi + (p ? n_pix : n_vis);
+        float h[3], l[3];
+        for (int d = 0; d < 3; ++d) {
+            h[d] = (float)xyz[d];
+            l[d] = (float)(xyz[d] - (double)h[d]);
+            m = fmaxf(m, fabsf(h[d]));
+        }
+        hi[k] = make_float4(h[0], h[1], h[2], 0.f);
+        lo[k] = make_float4(l[0], l[1], l[2], 0.f);
+        if (!p) V[k] = make_float2(0.f, 0.f);
     }
-    hi[i] = make_float4(h[0], h[1], h[2], 0.f);
-    lo[i] = make_float4(l[0], l[1], l[2], 0.f);
+    const unsigned bits = __float_as_uint(m);
+    const unsigned mp = __reduce_max_sync(0xffffffffu, p ? bits : 0u), mv = __reduce_max_sync(0xffffffffu, p ? 0u : bits);
+    if ((threadIdx.x & 31) == 0 && mp != 0u) atomicMax(top, mp);
+    if ((threadIdx.x & 31) == 0 && mv != 0u) atomicMax(top + 1, mv);
 }
 
-// The phase arithmetic and the two-level summation of direct_s2v_f32 (a register sum per
-// 256-pixel shared-memory tile, tile sums added with Kahan compensation); the baseline
-// tile comes from blockIdx.x and a segment of 4096 pixels from blockIdx.y instead of a
-// work list, and the segments' sums meet in V through atomicAdd, so their order (and the
-// last bits of the result) is not deterministic.
-__global__ void __launch_bounds__(kThreads) direct_s2v_f32_noalloc(
-    const float4 *__restrict__ vh, const float4 *__restrict__ vl, int n_vis, const float4 *__restrict__ rh_g,
-    const float4 *__restrict__ rl_g, const float *__restrict__ c, int n_pix, int seg, float2 *__restrict__ V,
-    float sgn) {
-    __shared__ float4 sh[kThreads];
-    __shared__ float4 sl[kThreads];
-    const int o0 = blockIdx.x * kTile, o1 = min(o0 + kTile, n_vis);
-    const int s_begin = blockIdx.y * seg, s_end = min(s_begin + seg, n_pix);
-    float3 ph[kPerThread], pl[kPerThread];
-    float are[kPerThread], aim[kPerThread], cre[kPerThread], cim[kPerThread];
-#pragma unroll
-    for (int v = 0; v < kPerThread; ++v) {
-        int k = o0 + threadIdx.x + v * kThreads;
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        if (k < o1) {
-            a = vh[k];
-            b = vl[k];
+// The FP32 direct sums (the wide form beyond the FP32 digits' reach) over items in a fixed order
+// instead of a work list; the segments' sums meet in V through atomicAdd, so their order (and
+// the last bits of the result) is not deterministic.
+template <class K>
+__device__ __forceinline__ void noalloc_items(const DirectJob &J, int n_vis, int n_pix, int seg, unsigned char *smem) {
+    DirectShared<K> &sh = *reinterpret_cast<DirectShared<K> *>(smem);
+    DirectPipe pipe = direct_begin(sh);
+    if constexpr (K::kMagnitudes)
+        for (int i = threadIdx.x; i < kDfTab; i += kDirectThreads) {
+            double sn, cs;
+            sincospi(2.0 * i / kDfTab, &sn, &cs);
+            const float ch = (float)cs, sh_ = (float)sn;
+            const float4 e = make_float4(ch, (float)(cs - (double)ch), sh_, (float)(sn - (double)sh_));
+            for (int c = 0; c < kDfCopies; ++c) sh.extra.e[i * kDfCopies + c] = e;
         }
-        ph[v] = make_float3(a.x, a.y, a.z);
-        pl[v] = make_float3(b.x, b.y, b.z);
-        are[v] = aim[v] = cre[v] = cim[v] = 0.f;
+    const int tiles = (n_vis + kRows - 1) / kRows, items = tiles * ((n_pix + seg - 1) / seg);
+    for (int it = blockIdx.x; it < items && !sh.abort; it += gridDim.x) {
+        const int o0 = it % tiles * kRows, s0 = it / tiles * seg;
+        direct_item<K, 0>(J, WorkItem{o0, min(o0 + kRows, n_vis), s0, min(s0 + seg, n_pix)}, sh, pipe);
+        __syncthreads();  // the owners' digits have had their last reader
     }
-    for (int s0 = s_begin; s0 < s_end; s0 += kThreads) {
-        __syncthreads();
-        int n = s0 + threadIdx.x;
-        if (n < s_end) {
-            float4 a = rh_g[n];
-            a.w = c[n];
-            sh[threadIdx.x] = a;
-            sl[threadIdx.x] = rl_g[n];
-        } else {
-            sh[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            sl[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-        const int cnt = min(kThreads, s_end - s0);
-        float tre[kPerThread], tim[kPerThread];
-#pragma unroll
-        for (int v = 0; v < kPerThread; ++v) tre[v] = tim[v] = 0.f;
-#pragma unroll 4
-        for (int q = 0; q < cnt; ++q) {
-            const float4 rh = sh[q], rl = sl[q];
-#pragma unroll
-            for (int v = 0; v < kPerThread; ++v) {
-                float f = phase_f32(ph[v], pl[v], rh, rl);
-                float sn, cs;
-                __sincosf(6.28318530717958648f * f, &sn, &cs);
-                tre[v] = __fmaf_rn(rh.w, cs, tre[v]);
-                tim[v] = __fmaf_rn(rh.w, sn, tim[v]);
-            }
-        }
-#pragma unroll
-        for (int v = 0; v < kPerThread; ++v) {
-            kahan_add(are[v], cre[v], tre[v]);
-            kahan_add(aim[v], cim[v], tim[v]);
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < kPerThread; ++v) {
-        int k = o0 + threadIdx.x + v * kThreads;
-        if (k < o1) {
-            atomicAdd(&V[k].x, __fsub_rn(are[v], cre[v]));
-            atomicAdd(&V[k].y, sgn * __fsub_rn(aim[v], cim[v]));
-        }
-    }
+    direct_end(sh, pipe);
+}
+
+__global__ void __launch_bounds__(kDirectThreads, 1)
+    direct_noalloc_kernel(DirectJob J, int n_vis, int n_pix, int seg, const unsigned *__restrict__ top) {
+    extern __shared__ __align__(128) unsigned char direct_smem[];
+    coord_scales(__uint_as_float(top[0]), J.pix_scale, J.vis_scale);
+    if (__uint_as_float(top[1]) * J.vis_scale <= kF32Reach)
+        noalloc_items<F32Kind<0>>(J, n_vis, n_pix, seg, direct_smem);
+    else
+        noalloc_items<DfKind<0, float>>(J, n_vis, n_pix, seg, direct_smem);
 }
 
 std::mutex g_noalloc_mu;
@@ -957,16 +945,19 @@ extern "C" hvox_status hvox_direct_synthesize_noalloc(const double *pix_xyz, int
         float4 *scratch = noalloc_scratch_for_current_device();
         float4 *rh = scratch, *rl = scratch + n_pix;
         float4 *vh = scratch + 2 * n_pix, *vl = vh + n_vis;
-        noalloc_split_kernel<<<(unsigned)((n_pix + 255) / 256), 256, 0, s>>>(pix_xyz, n_pix, rh, rl);
-        check_cuda(cudaGetLastError(), "noalloc_split pixels");
-        noalloc_split_kernel<<<(unsigned)((n_vis + 255) / 256), 256, 0, s>>>(uvw, n_vis, vh, vl);
-        check_cuda(cudaGetLastError(), "noalloc_split baselines");
-        check_cuda(cudaMemsetAsync(V, 0, sizeof(float) * 2 * (size_t)n_vis, s), "clear V");
-        const int seg = 4096;
-        dim3 grid((unsigned)((n_vis + kTile - 1) / kTile), (unsigned)((n_pix + seg - 1) / seg));
-        direct_s2v_f32_noalloc<<<grid, kThreads, 0, s>>>(vh, vl, (int)n_vis, rh, rl, I, (int)n_pix, seg,
-                                                          reinterpret_cast<float2 *>(V), (float)isign);
-        check_cuda(cudaGetLastError(), "direct_s2v_f32_noalloc");
+        unsigned *top = reinterpret_cast<unsigned *>(scratch + 2 * kNoAllocMaxPoints);
+        check_cuda(cudaMemsetAsync(top, 0, 2 * sizeof(unsigned), s), "clear coordinate maxima");
+        noalloc_prepare_kernel<<<(unsigned)((n_pix + n_vis + 255) / 256), 256, 0, s>>>(
+            pix_xyz, n_pix, uvw, n_vis, scratch, top, reinterpret_cast<float2 *>(V));
+        check_cuda(cudaGetLastError(), "noalloc_prepare");
+        const int64_t tiles = (n_vis + kRows - 1) / kRows;
+        const int64_t seg = direct_segment(tiles, n_pix), items = tiles * ((n_pix + seg - 1) / seg);
+        const DirectJob J{vh, vl, rh, rl, I, V, (float)isign, 1.f, 1.f, nullptr};
+        constexpr size_t smem = sizeof(DirectShared<DfKind<0, float>>);
+        static_assert(smem >= sizeof(DirectShared<F32Kind<0>>), "either form");
+        allow_smem<DirectJob>(direct_noalloc_kernel, smem);
+        direct_noalloc_kernel<<<grid_for(items, 1), kDirectThreads, smem, s>>>(J, (int)n_vis, (int)n_pix, (int)seg, top);
+        check_cuda(cudaGetLastError(), "direct_noalloc");
         set_error("");
         return HVOX_OK;
     } catch (const Error &e) {
