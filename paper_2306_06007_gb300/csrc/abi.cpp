@@ -200,9 +200,10 @@ constexpr double kDoubleFloatMinEps = 1e-9;
 constexpr double kDfftMinEps = 1e-11;
 bool dfft_wanted(int prec, bool plain, double eps) { return prec == 2 && !plain && eps >= kDfftMinEps; }
 
-// HVOX_DF_FFT=0 runs the same plan's FP64 grids through cuFFT Z2Z instead (comparisons).
-bool dfft_switched_off() {
-    const char *v = std::getenv("HVOX_DF_FFT");
+// HVOX_DF_FFT=0 runs the same plan's FP64 grids through cuFFT Z2Z instead, HVOX_C_FFT=0 its FP32
+// grids through the deconvolution passes and cuFFT C2C (comparisons).
+bool switched_off(const char *name) {
+    const char *v = std::getenv(name);
     return v && std::atoi(v) == 0;
 }
 
@@ -605,7 +606,8 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
         // selects full 3-D plans instead of the pruned pair.
         bool prune = true;
         if (const char *v = std::getenv("HVOX_FFT_PRUNE")) prune = std::atoi(v) != 0;
-        const bool use_dfft = dfft_wanted(p.prec, p.plain, p.eps) && !dfft_switched_off();
+        const bool use_dfft = dfft_wanted(p.prec, p.plain, p.eps) && !switched_off("HVOX_DF_FFT");
+        const bool use_cfft = p.prec == 1 && !p.plain && !switched_off("HVOX_C_FFT");
         std::vector<size_t> max_ws(n_lanes, 0);
         auto make = [&](cufftHandle &h, int rank, long long *n, long long *emb, long long stride, long long dist,
                         long long batch, size_t &ws) {
@@ -623,6 +625,19 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
         // grids of every wave share one format after the FFT.
         p.df_grids = use_dfft && prune;
         for (const NufftBlock &bk : part.blocks) p.df_grids = p.df_grids && dfft_supported(bk.n2);
+        p.cf_grids = use_cfft && prune;
+        for (const NufftBlock &bk : part.blocks) p.cf_grids = p.cf_grids && cfft_supported(bk.n2);
+        // A twiddle table of one length, shared by the plan's batches.
+        auto twiddles = [&](int n, auto make_table) -> void * {
+            auto &tab = p.fft_tw[n];
+            if (!tab) {
+                std::vector<float> t;
+                make_table(n, t);
+                tab = std::make_unique<DevBuf>();
+                upload(*tab, t.data(), t.size() * sizeof(float), s);
+            }
+            return tab->ptr;
+        };
         p.dblocks.resize(order.size());
         for (Wave &w : p.waves) {
             Lane &lane = *p.lanes[w.lane];
@@ -647,18 +662,24 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
                     for (int q = 0; q < 3; ++q) {
                         const int n = (int)fb.n2[q];
                         dfft_factor(n, *dd[q]);
-                        auto &tab = p.dfft_tw[n];
-                        if (!tab) {
-                            std::vector<float> t;
-                            dfft_twiddles(n, t);
-                            tab = std::make_unique<DevBuf>();
-                            upload(*tab, t.data(), t.size() * sizeof(float), s);
-                        }
-                        dd[q]->tw = tab->as<float4>();
+                        dd[q]->tw = static_cast<const float4 *>(twiddles(n, dfft_twiddles));
+                    }
+                }
+                // FP32 grids: the FP32 FFT where it covers every shape of the plan.
+                fb.cf = p.cf_grids;
+                fb.first = w.b0 + k;
+                for (int d = 0; d < 3; ++d) fb.n1[d] = first.n1[d];
+                if (fb.cf) {
+                    if (fault_hit("cufft")) fail(HVOX_ECUDA, "FP32 FFT plan: FFT error (injected)");
+                    CfftDev *cc[3] = {&fb.cx, &fb.cy, &fb.cz};
+                    for (int q = 0; q < 3; ++q) {
+                        const int n = (int)fb.n2[q];
+                        cfft_factor(n, *cc[q]);
+                        cc[q]->tw = static_cast<const float4 *>(twiddles(n, cfft_twiddles));
                     }
                 }
                 auto key = std::make_tuple(fb.n2[0], fb.n2[1], fb.n2[2], prune ? fb.half : (int64_t)-1, (int64_t)K);
-                if (!fb.df && !lane.fft.count(key)) {
+                if (!fb.df && !fb.cf && !lane.fft.count(key)) {
                     FftPlans &f = lane.fft[key];
                     size_t ws = 0;
                     if (prune) {
@@ -674,7 +695,7 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
                     }
                     max_ws[w.lane] = std::max(max_ws[w.lane], ws);
                 }
-                if (!fb.df) fb.plans = lane.fft[key];
+                if (!fb.df && !fb.cf) fb.plans = lane.fft[key];
                 w.ffts.push_back(fb);
                 for (int g = 0; g < K; ++g, ++k) {
                     const NufftBlock &bk = part.blocks[order[w.b0 + k]];
@@ -744,7 +765,7 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
                       &p.vis_lo, &p.items_s2v, &p.items_v2s, &p.item_counter, &p.inv_psi, &p.cheb, &p.src, &p.acc, &p.cis_tab, &p.err})
         ws += (double)b->bytes;
     for (auto &l : p.lanes) ws += (double)(l->g1.bytes + l->g2.bytes + l->work.bytes);
-    for (auto &kv : p.dfft_tw) ws += (double)kv.second->bytes;
+    for (auto &kv : p.fft_tw) ws += (double)kv.second->bytes;
     p.workspace_bytes = ws;
     p.plan_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
 }

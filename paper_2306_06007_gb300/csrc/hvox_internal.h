@@ -36,7 +36,7 @@ void check_cufft(cufftResult r, const char *what);
 // event of each named site (counted from the moment the variable last changed) fail the
 // way the real failure would:
 //   alloc    a device allocation (HVOX_ENOMEM, everything allocated so far freed);
-//   cufft    a cuFFT plan creation (HVOX_ECUDA);
+//   cufft    an FFT plan creation, cuFFT's or of the library's own FP32 FFT (HVOX_ECUDA);
 //   capture  a CUDA-graph capture (the plan falls back to eager launches);
 //   window   the pixel scale of the NUFFT sub-problem with the most pixels is multiplied
 //            by 4 on the host, so its kernels clamp the pixels' windows into the grid and
@@ -275,6 +275,19 @@ struct DfftDev {
     const float4 *tw = nullptr;
 };
 
+// One length of the FP32 FFT (k_cfft.cu): radices of its Stockham stages, the divisor of each stage's
+// butterfly index as a multiplier (as in DfftDev) and its twiddle tables.
+constexpr int kCfftMaxStages = 6;
+struct CfftDev {
+    int n = 0, stages = 0;
+    int radix[kCfftMaxStages] = {0};
+    unsigned ns_magic[kCfftMaxStages] = {0};
+    int tw_at[kCfftMaxStages] = {0};  // first float4 of each stage's twiddles
+    int pad = 0;                      // cells of padding per radix[0] elements in shared memory
+    unsigned r0_magic = 0;
+    const float4 *tw = nullptr;
+};
+
 // The batched transforms of K sub-problems of one grid shape inside a wave: their FFT
 // grids interleave z planes (plane z of grid g at g2 + (z K + g) * n2x n2y), so that each
 // band slab of all K grids is one contiguous run of planes (one batched 2-D call) and
@@ -289,6 +302,11 @@ struct FftBatch {
                               // (FP64 cells in, double-float cells out: Plan::df_grids)
     DfftDev dx, dy, dz;       // its three lengths
     int64_t h1y = 0;          // n1y / 2: the band rows are [0, h1y) and [n2y - h1y, n2y)
+    bool cf = false;          // FP32 grids through the library's FP32 FFT, which takes the
+                              // deconvolution passes along (Plan::cf_grids)
+    CfftDev cx, cy, cz;       // its three lengths
+    int64_t n1[3] = {0, 0, 0};
+    int first = 0;            // descriptor of the batch's first sub-problem
 };
 
 // Double-float FFT (k_dffft.cu): radices of length n (false when a factor other than 2, 3,
@@ -298,6 +316,14 @@ bool dfft_factor(int n, DfftDev &d);
 bool dfft_supported(const int64_t n2[3]);
 void dfft_twiddles(int n, std::vector<float> &tab);
 int dfft_batch(const FftBatch &f, int sign, bool band_input, cudaStream_t s);
+
+// FP32 FFT (k_cfft.cu): the same for FP32 grids. cfft_batch also deconvolves and pads the n1
+// grids before the transform (s2v) or crops and deconvolves into them after it.
+bool cfft_factor(int n, CfftDev &d);
+bool cfft_supported(const int64_t n2[3]);
+void cfft_twiddles(int n, std::vector<float> &tab);
+int cfft_batch(const FftBatch &f, const NufftDev *descs, void *g1, void *g2, const float *ipsi, int sign, bool s2v,
+               cudaStream_t s);
 
 // A wave: sub-problems [b0, b0 + nb) of the plan's descriptor array, run together: one
 // clearing, spreading, deconvolution and interpolation launch each (a 2-D launch grid over
@@ -330,6 +356,8 @@ template <typename T> struct NufftArgs {
     // FP64 plans whose FFT grids go through the double-float FFT: after the FFT the grid
     // holds float pairs (float4 per cell), which the double-float gathers and crop read.
     bool df_grids = false;
+    // FP32 plans whose FFT goes through the library's own transforms (which deconvolve too).
+    bool cf_grids = false;
     // FP64 spreading into fixed-point tiles of 32-bit limbs (k_nufft.cu) instead of FP64
     // shared atomics.
     bool int_tile = false;
@@ -435,8 +463,9 @@ struct Plan {
     std::vector<NufftDev> dblocks;      // block descriptors (wave order)
     DevBuf ddescs;                      // the same descriptors on the device
     std::vector<Wave> waves;            // waves of blocks (launch order)
-    std::map<int, std::unique_ptr<DevBuf>> dfft_tw;  // twiddle tables of the double-float FFT
+    std::map<int, std::unique_ptr<DevBuf>> fft_tw;   // twiddle tables of the library's own FFT
     bool df_grids = false;              // every FFT batch double-float (NufftArgs::df_grids)
+    bool cf_grids = false;              // every FFT batch by the FP32 FFT (NufftArgs::cf_grids)
     bool int_tile = false;              // NufftArgs::int_tile
     DevBuf cis_tab;                     // exp(j 2 pi m / 2048) as float pairs (double-float path)
     DevBuf err;                         // int: device error word (kDevErr* bits), read by hvox_sync

@@ -1499,9 +1499,12 @@ template <typename T, int W> void set_smem_attrs() {
 // In-place transforms of one batch of FFT grids with sign dir. band_input: only the n1
 // band's z planes are nonzero (sky -> vis: 2-D transforms of those planes, then z);
 // otherwise only those planes are read afterwards (vis -> sky: z first, then 2-D).
-// Returns the number of cuFFT executions.
-template <typename T> int fft_batch(const FftBatch &f, int dir, bool band_input, cudaStream_t s) {
+// Returns the number of launches (cuFFT: executions).
+template <typename T>
+int fft_batch(const FftBatch &f, const NufftArgs<T> &a, void *g1, void *g2, int dir, bool band_input, cudaStream_t s) {
     if (f.df) return dfft_batch(f, dir, band_input, s);
+    if constexpr (sizeof(T) == 4)
+        if (f.cf) return cfft_batch(f, a.descs, g1, g2, a.ipsi, dir, band_input, s);
     auto exec = [&](cufftHandle h, void *g) {
         check_cufft(cufftSetStream(h, s), "cufftSetStream");
         if constexpr (sizeof(T) == 4)
@@ -1548,14 +1551,16 @@ void nufft_wave_s2v(const Wave &w, const NufftArgs<T> &a, void *g1, void *g2, co
 #undef CALL
     check_cuda(cudaGetLastError(), "spread_pix");
     hook.end(HVOX_STAGE_SPREAD, 1, s);
-    hook.begin(HVOX_STAGE_DECONV, s);
-    deconv_pad_kernel<T><<<dgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g1),
-                                                       static_cast<cplx_t<T> *>(g2), a.ipsi);
-    check_cuda(cudaGetLastError(), "deconv_pad");
-    hook.end(HVOX_STAGE_DECONV, 1, s);
+    if (!a.cf_grids) {
+        hook.begin(HVOX_STAGE_DECONV, s);
+        deconv_pad_kernel<T><<<dgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g1),
+                                                           static_cast<cplx_t<T> *>(g2), a.ipsi);
+        check_cuda(cudaGetLastError(), "deconv_pad");
+        hook.end(HVOX_STAGE_DECONV, 1, s);
+    }
     hook.begin(HVOX_STAGE_FFT, s);
     int n_fft = 0;
-    for (const FftBatch &f : w.ffts) n_fft += fft_batch<T>(f, a.isign < 0 ? CUFFT_FORWARD : CUFFT_INVERSE, true, s);
+    for (const FftBatch &f : w.ffts) n_fft += fft_batch<T>(f, a, g1, g2, a.isign < 0 ? CUFFT_FORWARD : CUFFT_INVERSE, true, s);
     hook.end(HVOX_STAGE_FFT, n_fft, s);
     hook.begin(HVOX_STAGE_INTERP, s);
     if constexpr (sizeof(T) == 8) {
@@ -1605,7 +1610,7 @@ void nufft_wave_v2s(const Wave &w, const NufftArgs<T> &a, void *g1, void *g2, co
     hook.begin(HVOX_STAGE_FFT, s);
     int n_fft = 0;
     for (const FftBatch &f : w.ffts)  // transpose: opposite sign
-        n_fft += fft_batch<T>(f, a.isign < 0 ? CUFFT_INVERSE : CUFFT_FORWARD, false, s);
+        n_fft += fft_batch<T>(f, a, g1, g2, a.isign < 0 ? CUFFT_INVERSE : CUFFT_FORWARD, false, s);
     hook.end(HVOX_STAGE_FFT, n_fft, s);
     if constexpr (sizeof(T) == 8) {
         if (a.df_grids) {
@@ -1625,11 +1630,13 @@ void nufft_wave_v2s(const Wave &w, const NufftArgs<T> &a, void *g1, void *g2, co
             return;
         }
     }
-    hook.begin(HVOX_STAGE_DECONV, s);
-    crop_deconv_kernel<T><<<cgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g2),
-                                                        static_cast<cplx_t<T> *>(g1), a.ipsi);
-    check_cuda(cudaGetLastError(), "crop_deconv");
-    hook.end(HVOX_STAGE_DECONV, 1, s);
+    if (!a.cf_grids) {
+        hook.begin(HVOX_STAGE_DECONV, s);
+        crop_deconv_kernel<T><<<cgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g2),
+                                                            static_cast<cplx_t<T> *>(g1), a.ipsi);
+        check_cuda(cudaGetLastError(), "crop_deconv");
+        hook.end(HVOX_STAGE_DECONV, 1, s);
+    }
     hook.begin(HVOX_STAGE_INTERP, s);
 #define CALL(W)                                                                                                   \
     interp_pix_kernel<T, W><<<igrid, 128, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g1), a.pix_hi,  \
