@@ -17,10 +17,13 @@
 //  * plain path: everything in FP64 (the reference form the optimised paths replace; also for
 //    |p_d r_d| above 2^33 turns).
 //
-// What bounds them: FP32 issue. A pair takes ~14 instructions at FP32 (2 on the sine unit at a
-// quarter rate, a bound of 16 cycles for 32 pairs) and ~42 in double-float (28 before and 73
-// before with the phase on the FP32 pipes). Measured on one GB300 over 52,812 pixels x 1,435,200
-// baselines: 1.9e12 pairs/s at FP32 (1.16e12 before) and 7.0e11 in double-float (4.7e11 before).
+// What bounds them: at FP32 the sine unit (two results a pair at 8 cycles for 32: 16 cycles of
+// the 20 that 32 pairs take), in double-float the FMA pipe (60% busy), the shared-memory pipe (63%)
+// and issue (64%) together. FMAs and adds go two to an instruction (f32x2) over two columns or over
+// a sum's two parts: they take the FMA pipe as long as two scalar ones but half the issue slots.
+// Measured on one GB300 over 52,812 pixels x 1,435,200 baselines, pairs/s: FP32 1.16e12 with the
+// phase on the FP32 pipes, 1.95e12 with it on the tensor cores, 2.05e12 with f32x2; double-float
+// 4.7e11, 7.1e11 and 8.2e11.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
@@ -74,6 +77,40 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 __device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
     e = __fsub_rn(b, __fsub_rn(s, a));
+}
+
+// Two floats in one instruction (f32x2): the same operations and roundings as two scalar ones, for half the
+// issue slots.
+__device__ __forceinline__ uint64_t bits(float2 a) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 floats(uint64_t a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)), "l"(bits(c)));
+    return floats(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)));
+    return floats(r);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)));
+    return floats(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)));
+    return floats(r);
 }
 
 // The offset for a tile whose term magnitudes sum to at most S: 2^(floor(log2 S) + 2) > 2 S
@@ -362,84 +399,68 @@ template <class K> __device__ __forceinline__ void direct_end(DirectShared<K> &s
 // sum of 1.5M positive values (a long baseline's visibility) by that times its total. One
 // column in six (j: the column) takes the next float above 2 pi instead, (1 + 1.04e-7) 2 pi, so that
 // the factor is 1 + 4.05e-8 on average and the mean error of the cosine vanishes.
-__device__ __forceinline__ void cis_f32(float A, float B, int j, float &cs, float &sn) {
-    const float k = j % 6 == 5 ? 6.28318595886230469f : 6.28318548202514648f;
-    const float n = tc::nearest(A, 0x1p-14f);
-    const float a = __fmaf_rn(n, -0x1p14f, A);
-    const float x = __fmaf_rn(a, k * 0x1p-14f, __fmul_rn(B, k * 0x1p-25f));
-    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(sn) : "f"(x));
-    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(cs) : "f"(x));
+// Two columns (j even and j + 1) at once.
+__device__ __forceinline__ void cis_f32(float2 A, float2 B, int j, float2 &e0, float2 &e1) {
+    constexpr float k0 = 6.28318548202514648f, k1 = 6.28318595886230469f;
+    const float2 k = make_float2(k0, (j + 1) % 6 == 5 ? k1 : k0);
+    const float2 M = both(0x1.8p23f * 0x1p14f);  // adding it rounds to whole turns, A being in units of 2^-14
+    const float2 a = sub2(A, sub2(add2(A, M), M));
+    const float2 x = fma2(a, make_float2(k.x * 0x1p-14f, k.y * 0x1p-14f), mul2(B, make_float2(k.x * 0x1p-25f, k.y * 0x1p-25f)));
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(e0.x) : "f"(x.x));
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(e0.y) : "f"(x.x));
+    asm("cos.approx.ftz.f32 %0, %1;" : "=f"(e1.x) : "f"(x.y));
+    asm("sin.approx.ftz.f32 %0, %1;" : "=f"(e1.y) : "f"(x.y));
 }
 
 struct NoExtra {};
 
-template <int DIR> struct F32Sum;
-template <> struct F32Sum<0> {
-    float re, im, cre, cim, tre, tim;
+// sky -> vis: c cos and c sin. vis -> sky: Re(V e^{-isign j 2 pi t}) = Vr cos + isign Vi sin, a sum each.
+template <int DIR> struct F32Sum {
+    float re, im, cre, cim;
+    float2 t;  // the tile's sums
     __device__ __forceinline__ void clear() { re = im = cre = cim = 0.f; }
     __device__ __forceinline__ void poison() { re = im = __int_as_float(0x7fc00000); }
-    __device__ __forceinline__ void begin(const float *) { tre = tim = 0.f; }
+    __device__ __forceinline__ void begin(const float *) { t = both(0.f); }
     template <int N>
-    __device__ __forceinline__ void chunk(const float (&d)[2][N], const float *c, int j0, const NoExtra &) {
+    __device__ __forceinline__ void chunk(const float (&d)[2][N], const float2 *c, int j0, const NoExtra &) {
 #pragma unroll
-        for (int j = 0; j < N; j += 4) {
+        for (int j = 0; j < N; j += 2) {
             const float4 v = *reinterpret_cast<const float4 *>(c + j);
-            const float cv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float cs, sn;
-                cis_f32(d[0][j + i], d[1][j + i], j0 + j + i, cs, sn);
-                tre = __fmaf_rn(cv[i], cs, tre);
-                tim = __fmaf_rn(cv[i], sn, tim);
-            }
+            float2 e0, e1;
+            cis_f32(make_float2(d[0][j], d[0][j + 1]), make_float2(d[1][j], d[1][j + 1]), j0 + j, e0, e1);
+            t = fma2(make_float2(v.x, v.y), e0, t);
+            t = fma2(make_float2(v.z, v.w), e1, t);
         }
     }
     __device__ __forceinline__ void end() {
-        kahan_add(re, cre, tre);
-        kahan_add(im, cim, tim);
-    }
-    __device__ __forceinline__ void store(const DirectJob &J, int k) const {
-        float2 *acc = static_cast<float2 *>(J.acc);
-        atomicAdd(&acc[k].x, __fsub_rn(re, cre));
-        atomicAdd(&acc[k].y, J.sgn * __fsub_rn(im, cim));
-    }
-};
-template <> struct F32Sum<1> {
-    float re, cre, tre;
-    __device__ __forceinline__ void clear() { re = cre = 0.f; }
-    __device__ __forceinline__ void poison() { re = __int_as_float(0x7fc00000); }
-    __device__ __forceinline__ void begin(const float *) { tre = 0.f; }
-    template <int N>
-    __device__ __forceinline__ void chunk(const float (&d)[2][N], const float2 *V, int j0, const NoExtra &) {
-#pragma unroll
-        for (int j = 0; j < N; j += 2) {
-            const float4 v = *reinterpret_cast<const float4 *>(V + j);
-            const float vr[2] = {v.x, v.z}, vi[2] = {v.y, v.w};
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                float cs, sn;
-                cis_f32(d[0][j + i], d[1][j + i], j0 + j + i, cs, sn);
-                // Re(V e^{-isign j 2 pi t}) = Vr cos + isign Vi sin
-                tre = __fmaf_rn(vr[i], cs, __fmaf_rn(vi[i], sn, tre));
-            }
+        if constexpr (DIR == 0) {
+            kahan_add(re, cre, t.x);
+            kahan_add(im, cim, t.y);
+        } else {
+            kahan_add(re, cre, t.x + t.y);
         }
     }
-    __device__ __forceinline__ void end() { kahan_add(re, cre, tre); }
     __device__ __forceinline__ void store(const DirectJob &J, int k) const {
-        atomicAdd(static_cast<float *>(J.acc) + k, __fsub_rn(re, cre));
+        if constexpr (DIR == 0) {
+            float2 *acc = static_cast<float2 *>(J.acc);
+            atomicAdd(&acc[k].x, __fsub_rn(re, cre));
+            atomicAdd(&acc[k].y, J.sgn * __fsub_rn(im, cim));
+        } else {
+            atomicAdd(static_cast<float *>(J.acc) + k, __fsub_rn(re, cre));
+        }
     }
 };
 
 template <int DIR> struct F32Kind {
     using Form = tc::F32Form;
-    using Val = std::conditional_t<DIR == 0, float, float2>;
+    using Val = float2;  // (c, c), or V with isign on its imaginary part
     using Sum = F32Sum<DIR>;
     using Extra = NoExtra;
     static constexpr int kN = 64;
     static constexpr bool kMagnitudes = false;
     static __device__ __forceinline__ Val load(const DirectJob &J, int n) {
         if constexpr (DIR == 0) {
-            return static_cast<const float *>(J.val)[n];
+            return both(static_cast<const float *>(J.val)[n]);
         } else {
             float2 v = static_cast<const float2 *>(J.val)[n];
             v.y *= J.sgn;
@@ -454,7 +475,7 @@ constexpr int kDfTab = 1024;   // entries per turn of the sine table
 constexpr int kDfCopies = 8;   // one copy of each entry per lane of a quarter warp
 
 struct DfTable {
-    float4 e[kDfTab * kDfCopies];  // entry m, copy c: (cos_h, cos_l, sin_h, sin_l) of 2 pi m / 1024
+    float4 e[kDfTab * kDfCopies];  // entry m, copy c: (cos_h, sin_h, cos_l, sin_l) of 2 pi m / 1024
 };
 
 // exp(j 2 pi f) as (reh + rel) + j (imh + iml), f = (A - 1.5 2^23) / 1024 + B 2^-20 + C1 2^-31 + C2 2^-42
@@ -462,86 +483,84 @@ struct DfTable {
 // table's hi parts, exact floats); the remainder x (in units of 2^-20 turn, |x| <= 2^9) is formed
 // exactly but for its last rounding (2^-36 turn) and rotates the entry through cos x - 1 =
 // -x^2/2, sin x = x - x^3/6 in plain float. tab: the shared address of this lane's copy of the table.
-__device__ __forceinline__ void cis_df(float A, float B, float C1, float C2, uint32_t tab, float &reh, float &rel,
-                                       float &imh, float &iml) {
-    const float tt = __fmaf_rn(__fmaf_rn(C1, 0x1p-11f, B), 0x1p-10f, A);  // 1.5 2^23 + entry
-    const float d = __fmaf_rn(__fsub_rn(tt, A), -1024.f, B);
-    const float x = __fmaf_rn(C2, 0x1p-22f, __fmaf_rn(C1, 0x1p-11f, d));
-    const uint32_t at = ((__float_as_uint(tt) & (kDfTab - 1)) * (16u * kDfCopies)) + tab;
-    float4 tb;
-    asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(tb.x), "=f"(tb.y), "=f"(tb.z), "=f"(tb.w) : "r"(at));
+// Two columns at once; eh, el: (re, im) of each.
+__device__ __forceinline__ void cis_df(float2 A, float2 B, float2 C1, float2 C2, uint32_t tab, float2 (&eh)[2], float2 (&el)[2]) {
+    const float2 tt = fma2(fma2(C1, both(0x1p-11f), B), both(0x1p-10f), A);  // 1.5 2^23 + entry
+    const float2 d = fma2(sub2(tt, A), both(-1024.f), B);
+    const float2 x = fma2(C2, both(0x1p-22f), fma2(C1, both(0x1p-11f), d));
     constexpr float k = 6.28318530717958648f * 0x1p-20f;
-    const float x2 = __fmul_rn(x, x);
-    const float cm = __fmul_rn(x2, -0.5f * k * k);
-    const float sx = __fmul_rn(x, __fmaf_rn(x2, -k * k * k / 6.0f, k));
-    reh = tb.x;
-    rel = __fmaf_rn(-tb.z, sx, __fmaf_rn(tb.x, cm, tb.y));
-    imh = tb.z;
-    iml = __fmaf_rn(tb.x, sx, __fmaf_rn(tb.z, cm, tb.w));
+    const float2 x2 = mul2(x, x);
+    const float2 cm = mul2(x2, both(-0.5f * k * k));
+    const float2 sx = mul2(x, fma2(x2, both(-k * k * k / 6.0f), both(k)));
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t at = ((__float_as_uint(i ? tt.y : tt.x) & (kDfTab - 1)) * (16u * kDfCopies)) + tab;
+        float2 l;
+        asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(eh[i].x), "=f"(eh[i].y), "=f"(l.x), "=f"(l.y) : "r"(at));
+        const float c = i ? cm.y : cm.x, s = i ? sx.y : sx.x;
+        el[i].x = __fmaf_rn(-eh[i].y, s, __fmaf_rn(eh[i].x, c, l.x));
+        el[i].y = __fmaf_rn(eh[i].x, s, __fmaf_rn(eh[i].y, c, l.y));
+    }
 }
 
 // Offset double-float accumulation of one streamed tile: h += (ch + cl)(eh + el). The running
 // high sum starts at a power of two M above twice the tile's sum of term magnitudes S, so
 // it stays in [M - S, M + S]: h - h' is exact, and the part of both products that the two
 // FMAs rounded off is recovered by FMAs on that difference and collected in l with cl eh.
-// At the tile's end h - M is exact (Sterbenz).
+// At the tile's end h - M is exact (Sterbenz). Two sums at once: the real and imaginary part of a
+// visibility, or the products with the real and with the imaginary part of V of a pixel.
 struct DfAcc {
-    float h, l, oh, ol;  // tile sum (offset by M) and running sum
-    __device__ __forceinline__ void mac(float ch, float cl, float eh, float el) {
-        const float s = __fmaf_rn(ch, el, __fmaf_rn(ch, eh, h));
-        float u = __fmaf_rn(ch, eh, __fsub_rn(h, s));
-        u = __fmaf_rn(cl, eh, __fmaf_rn(ch, el, u));
+    float2 h, l;  // tile sums (h offset by M)
+    __device__ __forceinline__ void mac(float2 ch, float2 cl, float2 eh, float2 el) {
+        const float2 s = fma2(ch, el, fma2(ch, eh, h));
+        float2 u = fma2(ch, eh, sub2(h, s));
+        u = fma2(cl, eh, fma2(ch, el, u));
         h = s;
-        l = __fadd_rn(l, u);
+        l = add2(l, u);
     }
 };
 
 template <int DIR, class T> struct DfSum {
-    static constexpr int kV = DIR == 0 ? 2 : 1;  // re and im, or one real sum
-    DfAcc a[kV];
-    float M;
-    __device__ __forceinline__ void clear() {
-#pragma unroll
-        for (int c = 0; c < kV; ++c) a[c].oh = a[c].ol = 0.f;
-    }
-    __device__ __forceinline__ void poison() { a[0].oh = a[kV - 1].oh = __int_as_float(0x7fc00000); }
+    DfAcc a;
+    float M, oh[2], ol[2];  // running sums
+    __device__ __forceinline__ void clear() { oh[0] = oh[1] = ol[0] = ol[1] = 0.f; }
+    __device__ __forceinline__ void poison() { oh[0] = oh[1] = __int_as_float(0x7fc00000); }
     __device__ __forceinline__ void begin(const float *red) {
         float S = 0.f;
 #pragma unroll
         for (int i = 0; i < kStream / 32; ++i) S += red[i];
         M = tile_offset(1.01f * S);
-#pragma unroll
-        for (int c = 0; c < kV; ++c) {
-            a[c].h = M;
-            a[c].l = 0.f;
-        }
+        a.h = both(M);
+        a.l = both(0.f);
     }
-    template <int N, class Val>
-    __device__ __forceinline__ void chunk(const float (&d)[4][N], const Val *v, int, const DfTable &table) {
+    template <int N>
+    __device__ __forceinline__ void chunk(const float (&d)[4][N], const float4 *v, int, const DfTable &table) {
         const uint32_t tab = tc::smem_addr(&table.e[threadIdx.x & (kDfCopies - 1)]);
 #pragma unroll
-        for (int j = 0; j < N; ++j) {
-            float reh, rel, imh, iml;
-            cis_df(d[0][j], d[1][j], d[2][j], d[3][j], tab, reh, rel, imh, iml);
-            if constexpr (DIR == 0) {
-                const float2 c = v[j];
-                a[0].mac(c.x, c.y, reh, rel);
-                a[kV - 1].mac(c.x, c.y, imh, iml);
-            } else {
-                const float4 c = v[j];
-                a[0].mac(c.x, c.y, reh, rel);
-                a[0].mac(c.z, c.w, imh, iml);
+        for (int j = 0; j < N; j += 2) {
+            float2 eh[2], el[2];
+            cis_df(make_float2(d[0][j], d[0][j + 1]), make_float2(d[1][j], d[1][j + 1]), make_float2(d[2][j], d[2][j + 1]),
+                   make_float2(d[3][j], d[3][j + 1]), tab, eh, el);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const float4 c = v[j + i];
+                a.mac(make_float2(c.x, c.y), make_float2(c.z, c.w), eh[i], el[i]);
             }
         }
     }
     __device__ __forceinline__ void end() {
-#pragma unroll
-        for (int c = 0; c < kV; ++c) df_fold(a[c].oh, a[c].ol, __fsub_rn(a[c].h, M), a[c].l);
+        df_fold(oh[0], ol[0], __fsub_rn(a.h.x, M), a.l.x);
+        df_fold(oh[1], ol[1], __fsub_rn(a.h.y, M), a.l.y);
     }
     __device__ __forceinline__ void store(const DirectJob &J, int k) const {
-        T *acc = static_cast<T *>(J.acc) + (size_t)k * kV;
-        atomicAdd(acc, (T)((double)a[0].oh + (double)a[0].ol));
-        if constexpr (DIR == 0) atomicAdd(acc + 1, (T)((double)J.sgn * ((double)a[1].oh + (double)a[1].ol)));
+        const double re = (double)oh[0] + (double)ol[0], im = (double)oh[1] + (double)ol[1];
+        T *acc = static_cast<T *>(J.acc) + (size_t)k * (DIR == 0 ? 2 : 1);
+        if constexpr (DIR == 0) {
+            atomicAdd(acc, (T)re);
+            atomicAdd(acc + 1, (T)((double)J.sgn * im));
+        } else {
+            atomicAdd(acc, (T)(re + im));
+        }
     }
 };
 
@@ -550,27 +569,26 @@ template <int DIR, class T> struct DfSum {
 // T: the plan's real type (float: the wide path).
 template <int DIR, class T> struct DfKind {
     using Form = tc::DfForm;
-    using Val = std::conditional_t<DIR == 0, float2, float4>;
+    using Val = float4;  // (c_h, c_h, c_l, c_l), or (Vr_h, Vi_h, Vr_l, Vi_l) with isign on Vi
     using Sum = DfSum<DIR, T>;
     using Extra = DfTable;
     static constexpr int kN = 32;
     static constexpr bool kMagnitudes = true;
-    // (c_h, c_l), or (Vr_h, Vr_l, Vi_h, Vi_l) with isign on Vi
     static __device__ __forceinline__ Val load(const DirectJob &J, int n) {
         const T *v = static_cast<const T *>(J.val) + (size_t)n * (DIR == 0 ? 1 : 2);
         const float rh = (float)v[0], rl = (float)(v[0] - (T)rh);
         if constexpr (DIR == 0) {
-            return make_float2(rh, rl);
+            return make_float4(rh, rh, rl, rl);
         } else {
             const T vi = (T)J.sgn * v[1];
             const float ih = (float)vi;
-            return make_float4(rh, rl, ih, (float)(vi - (T)ih));
+            return make_float4(rh, ih, rl, (float)(vi - (T)ih));
         }
     }
     // each pair adds at most |c| or |Vr| + |Vi| to a sum
     static __device__ __forceinline__ float magnitude(const Val &v) {
         if constexpr (DIR == 0) return fabsf(v.x);
-        else return fabsf(v.x) + fabsf(v.z);
+        else return fabsf(v.x) + fabsf(v.y);
     }
 };
 
@@ -583,7 +601,10 @@ __global__ void __launch_bounds__(kDirectThreads, 1)
     DirectShared<K> &sh = *reinterpret_cast<DirectShared<K> *>(direct_smem);
     DirectPipe pipe = direct_begin(sh);
     if constexpr (K::kMagnitudes)
-        for (int i = threadIdx.x; i < kDfTab * kDfCopies; i += kDirectThreads) sh.extra.e[i] = gT[2 * (i / kDfCopies)];
+        for (int i = threadIdx.x; i < kDfTab * kDfCopies; i += kDirectThreads) {
+            const float4 e = gT[2 * (i / kDfCopies)];
+            sh.extra.e[i] = make_float4(e.x, e.z, e.y, e.w);
+        }
     for (int it = blockIdx.x; it < n_items && !sh.abort; it = next_item(counter, sh.next))
         direct_item<K, DIR>(job_of<BATCH>(J0, jobs, item_job, it), items[it], sh, pipe);
     direct_end(sh, pipe);
@@ -875,7 +896,7 @@ __device__ __forceinline__ void noalloc_items(const DirectJob &J, int n_vis, int
             double sn, cs;
             sincospi(2.0 * i / kDfTab, &sn, &cs);
             const float ch = (float)cs, sh_ = (float)sn;
-            const float4 e = make_float4(ch, (float)(cs - (double)ch), sh_, (float)(sn - (double)sh_));
+            const float4 e = make_float4(ch, sh_, (float)(cs - (double)ch), (float)(sn - (double)sh_));
             for (int c = 0; c < kDfCopies; ++c) sh.extra.e[i * kDfCopies + c] = e;
         }
     const int tiles = (n_vis + kRows - 1) / kRows, items = tiles * ((n_pix + seg - 1) / seg);
