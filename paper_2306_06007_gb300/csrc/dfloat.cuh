@@ -7,6 +7,8 @@
 
 #include <cuda_runtime.h>
 
+#include "f32x2.cuh"
+
 namespace hvox {
 namespace df {
 
@@ -78,6 +80,25 @@ __device__ __forceinline__ DF dmul2(DF a, DF b, DF c, DF d, float sg) {
     float s, t;
     fast_two_sum(r.h, r.l, s, t);
     return {s, t};
+}
+
+// Two double-floats (the real and imaginary part of a complex value) in packed instructions.
+struct DF2 {
+    float2 h, l;
+};
+__device__ __forceinline__ DF2 dneg2(DF2 a) { return {make_float2(-a.h.x, -a.h.y), make_float2(-a.l.x, -a.l.y)}; }
+
+// a w for a real w as an unnormalised p - ne (dmul_raw on both parts); na = -a.
+__device__ __forceinline__ void dscale_raw(DF2 a, DF2 na, DF w, float2 &p, float2 &ne) {
+    const float2 wh = f32x2::both(w.h), wl = f32x2::both(w.l);
+    p = f32x2::mul2(a.h, wh);
+    ne = f32x2::fma2(na.l, wh, f32x2::fma2(na.h, wl, f32x2::fma2(na.h, wh, p)));
+}
+__device__ __forceinline__ DF2 dscale(DF2 a, DF w) {
+    float2 p, ne;
+    dscale_raw(a, dneg2(a), w, p, ne);
+    const float2 s = f32x2::sub2(p, ne);
+    return {s, f32x2::sub2(f32x2::sub2(p, s), ne)};  // fast_two_sum(p, -ne)
 }
 
 // Lazy sum of several double-float terms with one renormalisation at the end: s is the

@@ -31,12 +31,15 @@
 #include <string>
 #include <type_traits>
 
+#include "f32x2.cuh"
 #include "hvox_internal.h"
 #include "phase_tc.cuh"
 
 namespace hvox {
 
 namespace {
+
+using namespace f32x2;
 
 constexpr int kThreads = 256;
 constexpr int kPerThread = 2;
@@ -77,40 +80,6 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
 __device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
     e = __fsub_rn(b, __fsub_rn(s, a));
-}
-
-// Two floats in one instruction (f32x2): the same operations and roundings as two scalar ones, for half the
-// issue slots.
-__device__ __forceinline__ uint64_t bits(float2 a) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
-    return r;
-}
-__device__ __forceinline__ float2 floats(uint64_t a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
-    return r;
-}
-__device__ __forceinline__ float2 both(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)), "l"(bits(c)));
-    return floats(r);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)));
-    return floats(r);
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)));
-    return floats(r);
-}
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-    uint64_t r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(bits(a)), "l"(bits(b)));
-    return floats(r);
 }
 
 // The offset for a tile whose term magnitudes sum to at most S: 2^(floor(log2 S) + 2) > 2 S
