@@ -311,14 +311,14 @@ struct FftBatch {
 
 // Double-float FFT (k_dffft.cu): radices of length n (false when a factor other than 2, 3,
 // 5, 7 remains), whether a grid shape is covered, the twiddle table of a length, and the
-// batched pruned 3-D transform of one batch (sign -1 or +1; band_input as fft_batch).
+// batched 3-D transform of one batch (sign -1 or +1) with its deconvolution: the n1 grids (FP64)
+// into the n2 grids (s2v) or the n2 grids (FP64) into the n1 grids, float pairs in either case.
 bool dfft_factor(int n, DfftDev &d);
 bool dfft_supported(const int64_t n2[3]);
 void dfft_twiddles(int n, std::vector<float> &tab);
-int dfft_batch(const FftBatch &f, int sign, bool band_input, cudaStream_t s);
+int dfft_batch(const FftBatch &f, const NufftDev *descs, void *g1, const double *ipsi, int sign, bool s2v, cudaStream_t s);
 
-// FP32 FFT (k_cfft.cu): the same for FP32 grids. cfft_batch also deconvolves and pads the n1
-// grids before the transform (s2v) or crops and deconvolves into them after it.
+// FP32 FFT (k_cfft.cu): the same for FP32 grids.
 bool cfft_factor(int n, CfftDev &d);
 bool cfft_supported(const int64_t n2[3]);
 void cfft_twiddles(int n, std::vector<float> &tab);

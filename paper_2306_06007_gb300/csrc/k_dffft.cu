@@ -7,13 +7,17 @@
 // runs in shared memory on the FP32 pipes: Stockham auto-sorting stages of radix 4, 2, 3, 5
 // and 7 (the odd radices through the symmetric form X_k, X_{r-k} = A_k +- s i B_k, half the
 // multiplications of a plain DFT), with twiddles exp(2 pi i q / n) computed in FP64 on the
-// host and stored as float pairs. One pass per dimension transforms the grid in place; the
-// first reads FP64 cells, every pass writes float pairs (the same 16 bytes per cell):
-//   rows (x): one row per CTA, only the rows that the pruned transform needs;
-//   columns (y): two adjacent columns per CTA (32-byte sectors), every column of a plane;
-//   columns (z): 64 adjacent columns per CTA, the planes of a batch interleaved; these short
-//   transforms (two stages for most grids) read the grid in their first stage and write it
-//   in their last, so they need one shared buffer and one barrier.
+// host and stored as float pairs. One pass per dimension; each reads and writes only what the n1
+// band leaves (the grid is zero outside it before the transform, unread outside it after):
+//   rows (x): one band row per CTA, multiplied by 1/Psi and padded from the FP64 n1 grid on the way in
+//     (sky -> vis), or cropped into it and multiplied on the way out (vis -> sky);
+//   columns (y): two adjacent columns per CTA (32-byte sectors), every column of a band plane;
+//   columns (z): 64 adjacent columns per CTA, the planes of a batch interleaved.
+// A pass's first stage reads the grid and its last one writes it: two barriers and two trips
+// through shared memory less than staging the whole sequence, and no deconvolution pass. Measured
+// over both directions of a 2160 x 2240 x 28 grid with the band 1436 x 1472 x 16: FFT and deconvolution
+// 10.2 -> 8.7 ms. What bounds the passes: FP32 issue and its latency (rows and columns 60 to 66%
+// of the issue slots, 47% of the warps an SM can hold), not HBM.
 // Transforms are unnormalised, sign s = -1 or +1: X_k = sum_q x_q exp(s 2 pi i q k / n).
 #include <algorithm>
 #include <cmath>
@@ -68,19 +72,11 @@ __device__ __forceinline__ float4 load_f64(const double2 *p) {
     const DF re = split_bits(v.x), im = split_bits(v.y);
     return make_float4(re.h, re.l, im.h, im.l);
 }
-__device__ __forceinline__ void store_f64(double2 *p, float4 v) {
-    *p = make_double2(f2d_bits(v.x) + f2d_bits(v.y), f2d_bits(v.z) + f2d_bits(v.w));
-}
-
 // A grid cell in either format: FP64 (double2) or, between the passes of one transform, the
 // double-float form itself (float4 of the same 16 bytes; zero is all-zero bits in both).
 template <bool F64> __device__ __forceinline__ float4 load_cell(double2 *p) {
     if constexpr (F64) return load_f64(p);
     else return *reinterpret_cast<const float4 *>(p);
-}
-template <bool F64> __device__ __forceinline__ void store_cell(double2 *p, float4 v) {
-    if constexpr (F64) store_f64(p, v);
-    else *reinterpret_cast<float4 *>(p) = v;
 }
 
 // Twiddle exp(SG 2 pi i e / n) from the table of exp(2 pi i q / n) (cos h, cos l, sin h, sin l).
@@ -185,20 +181,59 @@ template <int TX> struct SmemSt {
     float4 *b;
     __device__ __forceinline__ void operator()(int e, int t, float4 v) const { b[e * TX + t] = v; }
 };
+// Elements outside the band [0, h) and [n - h, n) (gap = n - 2 h) read as zero and are not written.
+__device__ __forceinline__ bool in_band(int e, int h, int gap) { return (unsigned)(e - h) >= (unsigned)gap; }
 template <bool F64> struct ColLd {
     double2 *base;
     int64_t stride;
-    int valid;
+    int valid, h, gap;
     __device__ __forceinline__ float4 operator()(int e, int t) const {
-        return t < valid ? load_cell<F64>(base + e * stride + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        return t < valid && in_band(e, h, gap) ? load_cell<F64>(base + e * stride + t) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
 };
-template <bool F64> struct ColSt {
+struct ColSt {
     double2 *base;
     int64_t stride;
-    int valid;
+    int valid, h, gap;
     __device__ __forceinline__ void operator()(int e, int t, float4 v) const {
-        if (t < valid) store_cell<F64>(base + e * stride + t, v);
+        if (t < valid && in_band(e, h, gap)) *reinterpret_cast<float4 *>(base + e * stride + t) = v;
+    }
+};
+// A row of the n2 grid, and the row of the n1 grid it comes from (FP64, multiplied by 1/Psi and padded) or
+// goes to (float pairs, cropped and multiplied): band element e is n1 element e + h or e - h - gap.
+struct RowLd {
+    const double2 *row;
+    __device__ __forceinline__ float4 operator()(int e, int) const { return *reinterpret_cast<const float4 *>(row + e); }
+};
+struct RowSt {
+    double2 *row;
+    __device__ __forceinline__ void operator()(int e, int, float4 v) const { *reinterpret_cast<float4 *>(row + e) = v; }
+};
+struct BandLd {
+    const double2 *in;
+    const double *px;
+    double fyz;
+    int h, gap;
+    __device__ __forceinline__ float4 operator()(int e, int) const {
+        if (!in_band(e, h, gap)) return make_float4(0.f, 0.f, 0.f, 0.f);
+        const int i = e < h ? e + h : e - h - gap;
+        const double2 g = in[i];
+        const double f = px[i] * fyz;
+        const DF re = split_bits(g.x * f), im = split_bits(g.y * f);
+        return make_float4(re.h, re.l, im.h, im.l);
+    }
+};
+struct BandSt {
+    float4 *out;
+    const double *px;
+    double fyz;
+    int h, gap;
+    __device__ __forceinline__ void operator()(int e, int, float4 v) const {
+        if (!in_band(e, h, gap)) return;
+        const int i = e < h ? e + h : e - h - gap;
+        const DF f = split_bits(px[i] * fyz);
+        const DF re = dmul({v.x, v.y}, f), im = dmul({v.z, v.w}, f);
+        out[i] = make_float4(re.h, re.l, im.h, im.l);
     }
 };
 
@@ -242,75 +277,53 @@ __device__ __forceinline__ void fft_pass(float4 *a, float4 *b, const DfftDev &d,
 // Shared buffers a pass needs for a transform of s stages (see fft_pass).
 inline int pass_buffers(int s) { return s >= 3 ? 2 : s - 1; }
 
-// In-place transforms of TX interleaved sequences of length n in shared memory (element q of
-// sequence t at a[q TX + t]); b is the second buffer of the Stockham ping-pong. Returns the
-// buffer holding the result.
-template <int TX, int SG>
-__device__ float4 *fft_smem(float4 *a, float4 *b, const DfftDev &d) {
-    int Ns = 1;
-    for (int st = 0; st < d.stages; ++st) {
-        run_stage<TX, SG>(d.radix[st], SmemLd<TX>{a}, SmemSt<TX>{b}, d, Ns, d.ns_magic[st]);
-        __syncthreads();
-        float4 *tmp = a;
-        a = b;
-        b = tmp;
-        Ns *= d.radix[st];
-    }
-    return a;
-}
-
 // Linear index of a band plane (the n1 band's z planes of a batch: the lower slab's
 // half K planes, then the upper slab's) -> plane number in the interleaved layout.
 __device__ __forceinline__ int64_t band_plane(int64_t P, int64_t halfK, int64_t n2z, int64_t K, int64_t half) {
     return P < halfK ? P : (n2z - half) * K + (P - halfK);
 }
 
-// Rows (x): sequence s = (band plane P, row R) with R over all n2y rows or only the band rows.
-// IN64 / OUT64: the grid holds FP64 values before / after the pass (else double-float).
-template <int SG, bool IN64, bool OUT64>
-__global__ void __launch_bounds__(kFftThreads, 4) dfft_rows_kernel(double2 *__restrict__ g, DfftDev d, int64_t n2y,
-                                                                 int64_t halfK, int64_t n2z, int64_t K, int64_t half,
-                                                                 int64_t rows, int64_t h1y) {
+// Rows (x): sequence s = (band plane P, band row R), R < 2 h1y. OUT false: n1 grid -> n2 rows, true: n2 rows ->
+// n1 grid.
+template <int SG, bool OUT>
+__global__ void __launch_bounds__(kFftThreads, 4)
+    dfft_rows_kernel(double2 *__restrict__ g, DfftDev d, int n2y, int n2z, int K, int h1x, int h1y, int h1z,
+                     const NufftDev *__restrict__ descs, void *__restrict__ g1, const double *__restrict__ ipsi) {
     extern __shared__ float4 smem[];
-    const int n = d.n;
-    const int64_t s = blockIdx.x;
-    const int64_t P = s / rows, R = s - P * rows;
-    const int64_t y = h1y > 0 ? (R < h1y ? R : n2y - h1y + (R - h1y)) : R;
-    double2 *row = g + (band_plane(P, halfK, n2z, K, half) * n2y + y) * n;
-    float4 *a = smem, *b = smem + n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) a[i] = load_cell<IN64>(row + i);
-    __syncthreads();
-    const float4 *out = fft_smem<1, SG>(a, b, d);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) store_cell<OUT64>(row + i, out[i]);
+    const int n = d.n, rows = 2 * h1y;
+    const int64_t P = blockIdx.x / rows;
+    const int R = (int)(blockIdx.x - P * rows);
+    const int iz2 = (int)(P / K), grid = (int)(P - (int64_t)iz2 * K);  // lower slab, then upper slab
+    const int jz = iz2 < h1z ? iz2 : n2z - 2 * h1z + iz2, jy = R < h1y ? R : n2y - rows + R;
+    const int iz = iz2 < h1z ? iz2 + h1z : iz2 - h1z, iy = R < h1y ? R + h1y : R - h1y;
+    const NufftDev &b = descs[grid];
+    const double *px = ipsi + b.psi_off, *py = px + 2 * h1x, *pz = py + rows;
+    const double fyz = py[iy] * pz[iz];
+    const int64_t band = b.g1_off + ((int64_t)iz * rows + iy) * 2 * h1x;
+    double2 *row = g + (((int64_t)jz * K + grid) * n2y + jy) * n;
+    if constexpr (OUT)
+        fft_pass<1, SG>(smem, smem + n, d, RowLd{row}, BandSt{static_cast<float4 *>(g1) + band, px, fyz, h1x, n - 2 * h1x});
+    else
+        fft_pass<1, SG>(smem, smem + n, d, BandLd{static_cast<const double2 *>(g1) + band, px, fyz, h1x, n - 2 * h1x}, RowSt{row});
 }
 
 // Columns: TX adjacent columns starting at column c0 of a plane (y: columns of one band plane,
 // stride n2x; z: every column of the batch, stride K n2x n2y), element q at c + q * stride.
-template <int TX, int SG, bool IN64, bool OUT64>
+// (hi, gi): band of the input, (ho, go): of the output.
+struct ColBands {
+    int hi, gi, ho, go;
+};
+template <int TX, int SG, bool IN64>
 __global__ void __launch_bounds__(kFftThreads, 4) dfft_cols_kernel(double2 *__restrict__ g, DfftDev d, int64_t stride,
                                                                  int64_t ncols, int64_t plane_cells, int64_t halfK,
-                                                                 int64_t n2z, int64_t K, int64_t half, int band) {
+                                                                 int64_t n2z, int64_t K, int64_t half, int band, ColBands b) {
     extern __shared__ float4 smem[];
-    const int n = d.n;
     const int64_t tiles = (ncols + TX - 1) / TX;
     const int64_t P = blockIdx.x / tiles, c0 = (blockIdx.x - P * tiles) * TX;
     double2 *base = g + (band ? band_plane(P, halfK, n2z, K, half) * plane_cells : 0) + c0;
     const int valid = ncols - c0 < TX ? (int)(ncols - c0) : TX;
-    float4 *a = smem, *b = smem + (size_t)n * TX;
-    if constexpr (TX == 64) {  // the short z columns: first and last stage on the grid
-        fft_pass<TX, SG>(a, b, d, ColLd<IN64>{base, stride, valid}, ColSt<OUT64>{base, stride, valid});
-    } else {
-        for (int e = threadIdx.x; e < n * TX; e += blockDim.x) {
-            const int q = e / TX, t = e - q * TX;
-            a[e] = t < valid ? load_cell<IN64>(base + q * stride + t) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-        const float4 *out = fft_smem<TX, SG>(a, b, d);
-        for (int e = threadIdx.x; e < n * TX; e += blockDim.x) {
-            const int q = e / TX, t = e - q * TX;
-            if (t < valid) store_cell<OUT64>(base + q * stride + t, out[e]);
-        }
-    }
+    fft_pass<TX, SG>(smem, smem + (size_t)d.n * TX, d, ColLd<IN64>{base, stride, valid, b.hi, b.gi},
+                     ColSt{base, stride, valid, b.ho, b.go});
 }
 
 constexpr size_t kFftSmemMax = 220 * 1024;
@@ -320,18 +333,14 @@ template <typename K> void allow_smem(K kernel) {
                "cudaFuncSetAttribute");
 }
 
-// Cell formats of a pass: kDD double-float in and out, kFD FP64 in, kDF FP64 out.
-enum Io { kDD = 0, kFD = 1, kDF = 2 };
-
 template <int TX, int SG> void allow_cols() {
-    allow_smem(dfft_cols_kernel<TX, SG, false, false>);
-    allow_smem(dfft_cols_kernel<TX, SG, true, false>);
-    allow_smem(dfft_cols_kernel<TX, SG, false, true>);
+    allow_smem(dfft_cols_kernel<TX, SG, false>);
+    allow_smem(dfft_cols_kernel<TX, SG, true>);
 }
 
 template <int SG> void allow_sign() {
-    allow_smem(dfft_rows_kernel<SG, true, false>);
-    allow_smem(dfft_rows_kernel<SG, false, false>);
+    allow_smem(dfft_rows_kernel<SG, true>);
+    allow_smem(dfft_rows_kernel<SG, false>);
     allow_cols<1, SG>();
     allow_cols<2, SG>();
     allow_cols<8, SG>();
@@ -354,49 +363,23 @@ int cols_per_cta(int n, int want) {
     return 0;
 }
 
-template <int TX, int SG, bool IN64, bool OUT64>
-void launch_cols(double2 *g, const DfftDev &d, int64_t stride, int64_t ncols, int64_t plane_cells, int64_t planes,
-                 int64_t halfK, int64_t n2z, int64_t K, int64_t half, int band, cudaStream_t s) {
+template <int TX, int SG>
+void launch_cols(bool in64, double2 *g, const DfftDev &d, int64_t stride, int64_t ncols, int64_t plane_cells, int64_t planes,
+                 int64_t halfK, int64_t n2z, int64_t K, int64_t half, int band, ColBands b, cudaStream_t s) {
     const int64_t tiles = (ncols + TX - 1) / TX;
-    const size_t smem = (size_t)(TX == 64 ? pass_buffers(d.stages) : 2) * d.n * TX * sizeof(float4);
-    dfft_cols_kernel<TX, SG, IN64, OUT64><<<(unsigned)(planes * tiles), kFftThreads, smem, s>>>(
-        g, d, stride, ncols, plane_cells, halfK, n2z, K, half, band);
+    const size_t smem = (size_t)pass_buffers(d.stages) * d.n * TX * sizeof(float4);
+    const auto kernel = in64 ? dfft_cols_kernel<TX, SG, true> : dfft_cols_kernel<TX, SG, false>;
+    kernel<<<(unsigned)(planes * tiles), kFftThreads, smem, s>>>(g, d, stride, ncols, plane_cells, halfK, n2z, K, half, band, b);
     check_cuda(cudaGetLastError(), "dfft_cols");
 }
 
-template <int TX, int SG>
-void launch_cols_io(Io io, double2 *g, const DfftDev &d, int64_t stride, int64_t ncols, int64_t plane_cells,
-                    int64_t planes, int64_t halfK, int64_t n2z, int64_t K, int64_t half, int band, cudaStream_t s) {
-    if (io == kFD) launch_cols<TX, SG, true, false>(g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s);
-    else if (io == kDF) launch_cols<TX, SG, false, true>(g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s);
-    else launch_cols<TX, SG, false, false>(g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s);
-}
-
-template <int SG>
-void cols_sign(int tx, Io io, double2 *g, const DfftDev &d, int64_t stride, int64_t ncols, int64_t plane_cells,
-               int64_t planes, int64_t halfK, int64_t n2z, int64_t K, int64_t half, int band, cudaStream_t s) {
+template <int SG, class... A> void cols_sign(int tx, A... a) {
     switch (tx) {
-        case 64: launch_cols_io<64, SG>(io, g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s); break;
-        case 8: launch_cols_io<8, SG>(io, g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s); break;
-        case 2: launch_cols_io<2, SG>(io, g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s); break;
-        default: launch_cols_io<1, SG>(io, g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s); break;
+        case 64: launch_cols<64, SG>(a...); break;
+        case 8: launch_cols<8, SG>(a...); break;
+        case 2: launch_cols<2, SG>(a...); break;
+        default: launch_cols<1, SG>(a...); break;
     }
-}
-
-void cols(int tx, Io io, double2 *g, const DfftDev &d, int64_t stride, int64_t ncols, int64_t plane_cells,
-          int64_t planes, int64_t halfK, int64_t n2z, int64_t K, int64_t half, int band, int sign, cudaStream_t s) {
-    if (sign > 0) cols_sign<1>(tx, io, g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s);
-    else cols_sign<-1>(tx, io, g, d, stride, ncols, plane_cells, planes, halfK, n2z, K, half, band, s);
-}
-
-template <int SG>
-void launch_rows(Io io, unsigned grid, size_t smem, double2 *g, const DfftDev &d, int64_t n2y, int64_t halfK,
-                 int64_t n2z, int64_t K, int64_t half, int64_t rows, int64_t h1y, cudaStream_t s) {
-    if (io == kFD)
-        dfft_rows_kernel<SG, true, false><<<grid, kFftThreads, smem, s>>>(g, d, n2y, halfK, n2z, K, half, rows, h1y);
-    else
-        dfft_rows_kernel<SG, false, false><<<grid, kFftThreads, smem, s>>>(g, d, n2y, halfK, n2z, K, half, rows, h1y);
-    check_cuda(cudaGetLastError(), "dfft_rows");
 }
 
 }  // namespace
@@ -452,38 +435,46 @@ void dfft_twiddles(int n, std::vector<float> &tab) {
     }
 }
 
-int dfft_batch(const FftBatch &f, int sign, bool band_input, cudaStream_t s) {
+int dfft_batch(const FftBatch &f, const NufftDev *descs, void *g1, const double *ipsi, int sign, bool s2v, cudaStream_t s) {
     set_fft_attrs();
     double2 *g = static_cast<double2 *>(f.g2);
     const int64_t n2x = f.n2[0], n2y = f.n2[1], n2z = f.n2[2], K = f.K, half = f.half;
     const int64_t halfK = half * K, band_planes = 2 * halfK, plane = n2x * n2y;
-    // The grid is FP64 before the first pass (written by the deconvolution or the spreading)
-    // and holds double-float values after it: the last pass leaves them for the
-    // double-float gathers (sky -> vis) or crop (vis -> sky).
-    auto rows = [&](Io io) {
-        const int64_t r = 2 * f.h1y;  // band rows only
-        const size_t smem = (size_t)2 * n2x * sizeof(float4);
-        const unsigned grid = (unsigned)(band_planes * r);
-        if (sign > 0) launch_rows<1>(io, grid, smem, g, f.dx, n2y, halfK, n2z, K, half, r, f.h1y, s);
-        else launch_rows<-1>(io, grid, smem, g, f.dx, n2y, halfK, n2z, K, half, r, f.h1y, s);
+    // The grids are FP64 before the first pass (written by the spreading) and hold double-float values
+    // after it: the last pass leaves them for the double-float gathers.
+    auto rows = [&] {
+        const size_t smem = (size_t)pass_buffers(f.dx.stages) * n2x * sizeof(float4);
+        const unsigned grid = (unsigned)(band_planes * f.n1[1]);
+        const auto kernel = sign > 0 ? (s2v ? dfft_rows_kernel<1, false> : dfft_rows_kernel<1, true>)
+                                     : (s2v ? dfft_rows_kernel<-1, false> : dfft_rows_kernel<-1, true>);
+        kernel<<<grid, kFftThreads, smem, s>>>(g, f.dx, (int)n2y, (int)n2z, (int)K, (int)(f.n1[0] / 2), (int)(f.n1[1] / 2),
+                                               (int)half, descs + f.first, g1, ipsi);
+        check_cuda(cudaGetLastError(), "dfft_rows");
     };
+    auto bands = [&](int64_t n, int64_t h) {  // the n1 band of the pass's input (sky -> vis) or output
+        const int hh = (int)h, gap = (int)(n - 2 * h);
+        return s2v ? ColBands{hh, gap, 0, 0} : ColBands{0, 0, hh, gap};
+    };
+    auto cols = [&](int tx, auto... a) { return sign > 0 ? cols_sign<1>(tx, a..., s) : cols_sign<-1>(tx, a..., s); };
     // y columns: two adjacent columns per CTA (32-byte segments) unless that leaves fewer than
     // two CTAs per SM (long columns), then one (twice the DRAM sectors, at ~15 % of HBM).
     const int ty = (size_t)2 * n2y * 2 * sizeof(float4) <= kFftSmemMax / 2 ? 2 : 1;
     auto ycols = [&] {
-        cols(cols_per_cta((int)n2y, ty), kDD, g, f.dy, n2x, n2x, plane, band_planes, halfK, n2z, K, half, 1, sign, s);
+        cols(cols_per_cta((int)n2y, ty), false, g, f.dy, n2x, n2x, plane, band_planes, halfK, n2z, K, half, 1,
+             bands(n2y, f.n1[1] / 2));
     };
-    auto zcols = [&](Io io) {
-        cols(cols_per_cta((int)n2z, 64), io, g, f.dz, K * plane, K * plane, 0, 1, halfK, n2z, K, half, 0, sign, s);
+    auto zcols = [&](bool in64) {
+        cols(cols_per_cta((int)n2z, 64), in64, g, f.dz, K * plane, K * plane, (int64_t)0, (int64_t)1, halfK, n2z, K, half, 0,
+             bands(n2z, half));
     };
-    if (band_input) {  // only the band rows of the band planes are nonzero
-        rows(kFD);
+    if (s2v) {  // only the band rows of the band planes are nonzero
+        rows();
         ycols();
-        zcols(kDD);
+        zcols(false);
     } else {  // only the band rows of the band planes are read afterwards
-        zcols(kFD);
+        zcols(true);
         ycols();
-        rows(kDD);
+        rows();
     }
     return 3;
 }

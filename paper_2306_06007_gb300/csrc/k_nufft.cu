@@ -1420,59 +1420,6 @@ __global__ void __launch_bounds__(kRowThreads) crop_deconv_kernel(const NufftDev
     }
 }
 
-// crop_deconv for double-float grids (after the double-float FFT): reads float-pair cells
-// of the n2 band, writes the n1 grid as float pairs for interp_pix_df_kernel; the
-// deconvolution factor is formed in FP64 once per cell and multiplied in double-float.
-__global__ void __launch_bounds__(kRowThreads) crop_deconv_df_kernel(const NufftDev *__restrict__ descs, int b0,
-                                                                     const float4 *__restrict__ G2base,
-                                                                     float4 *__restrict__ G1base,
-                                                                     const double *__restrict__ ipsi_all) {
-    __shared__ NufftDev sb;
-    load_desc(sb, descs + b0 + blockIdx.y);
-    const NufftDev &b = sb;
-    const int n1x = b.n1[0], n1y = b.n1[1], n1z = b.n1[2];
-    const int n2x = b.n2[0], n2y = b.n2[1], n2z = b.n2[2];
-    const double *ipsi = ipsi_all + b.psi_off;
-    const double *px = ipsi, *py = ipsi + n1x, *pz = py + n1y;
-    const float4 *G2 = G2base + b.g2_off;
-    float4 *G1 = G1base + b.g1_off;
-    int64_t r, cnt;
-    warp_rows((int64_t)n1y * n1z, r, cnt);
-    if (cnt == 0) return;
-    int iy = (int)(r % n1y), iz = (int)(r / n1y);
-    const int lane = threadIdx.x & 31;
-    for (int64_t k = 0; k < cnt; ++k) {
-        int jy = iy - n1y / 2, jz = iz - n1z / 2;
-        jy += jy < 0 ? n2y : 0;
-        jz += jz < 0 ? n2z : 0;
-        const float4 *in = G2 + (int64_t)jz * b.zs2 + (int64_t)jy * n2x;
-        float4 *out = G1 + ((int64_t)iz * n1y + iy) * n1x;
-        const double fyz = py[iy] * pz[iz];
-        for (int x0 = lane; x0 < n1x; x0 += 32 * kRowUnroll) {
-            float4 v[kRowUnroll];
-#pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
-                const int ix = x0 + 32 * u;
-                if (ix < n1x) {
-                    int jx = ix - n1x / 2;
-                    jx += jx < 0 ? n2x : 0;
-                    const float4 g = in[jx];
-                    const df::DF f = df::split_bits(px[ix] * fyz);
-                    const df::DF re = df::dmul({g.x, g.y}, f), im = df::dmul({g.z, g.w}, f);
-                    v[u] = make_float4(re.h, re.l, im.h, im.l);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u)
-                if (x0 + 32 * u < n1x) out[x0 + 32 * u] = v[u];
-        }
-        if (++iy == n1y) {
-            iy = 0;
-            ++iz;
-        }
-    }
-}
-
 #define HVOX_W_SWITCH(w, CALL)                                         \
     switch (w) {                                                       \
         case 2: CALL(2); break;                                        \
@@ -1520,7 +1467,8 @@ template <typename T, int W> void set_smem_attrs() {
 // Returns the number of launches (cuFFT: executions).
 template <typename T>
 int fft_batch(const FftBatch &f, const NufftArgs<T> &a, void *g1, void *g2, int dir, bool band_input, cudaStream_t s) {
-    if (f.df) return dfft_batch(f, dir, band_input, s);
+    if constexpr (sizeof(T) == 8)
+        if (f.df) return dfft_batch(f, a.descs, g1, a.ipsi, dir, band_input, s);
     if constexpr (sizeof(T) == 4)
         if (f.cf) return cfft_batch(f, a.descs, g1, g2, a.ipsi, dir, band_input, s);
     auto exec = [&](cufftHandle h, void *g) {
@@ -1569,7 +1517,7 @@ void nufft_wave_s2v(const Wave &w, const NufftArgs<T> &a, void *g1, void *g2, co
 #undef CALL
     check_cuda(cudaGetLastError(), "spread_pix");
     hook.end(HVOX_STAGE_SPREAD, 1, s);
-    if (!a.cf_grids) {
+    if (!a.cf_grids && !a.df_grids) {
         hook.begin(HVOX_STAGE_DECONV, s);
         deconv_pad_kernel<T><<<dgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g1),
                                                            static_cast<cplx_t<T> *>(g2), a.ipsi);
@@ -1632,11 +1580,6 @@ void nufft_wave_v2s(const Wave &w, const NufftArgs<T> &a, void *g1, void *g2, co
     hook.end(HVOX_STAGE_FFT, n_fft, s);
     if constexpr (sizeof(T) == 8) {
         if (a.df_grids) {
-            hook.begin(HVOX_STAGE_DECONV, s);
-            crop_deconv_df_kernel<<<cgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const float4 *>(g2),
-                                                                static_cast<float4 *>(g1), a.ipsi);
-            check_cuda(cudaGetLastError(), "crop_deconv_df");
-            hook.end(HVOX_STAGE_DECONV, 1, s);
             hook.begin(HVOX_STAGE_INTERP, s);
 #define CALL(W)                                                                                                   \
     interp_pix_df_kernel<W><<<igrid, 128, 0, s>>>(a.descs, w.b0, static_cast<const float4 *>(g1), a.pix_hi,      \
@@ -1648,7 +1591,7 @@ void nufft_wave_v2s(const Wave &w, const NufftArgs<T> &a, void *g1, void *g2, co
             return;
         }
     }
-    if (!a.cf_grids) {
+    if (!a.cf_grids && !a.df_grids) {
         hook.begin(HVOX_STAGE_DECONV, s);
         crop_deconv_kernel<T><<<cgrid, kRowThreads, 0, s>>>(a.descs, w.b0, static_cast<const cplx_t<T> *>(g2),
                                                             static_cast<cplx_t<T> *>(g1), a.ipsi);
