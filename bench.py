@@ -46,14 +46,10 @@ WORKLOAD = ("LOFAR-like: HEALPix nside=256 30deg cap (52,812 px) x 300 antennas 
 FP32_PEAK_FLOPS = 152 * 128 * 2 * 2.07e9  # FP32 FMA pipes x 2 flops x max SM clock
 FLOPS_PER_PAIR = 16.0                      # algorithmic flops per (pixel, baseline) pair
 
-# From ncu captures of the direct kernels on the LOFAR-like workload at eps = 1e-9, valid
-# only for the kernel source they were taken on: DRAM bytes per launch (dram__bytes_read.sum +
-# dram__bytes_write.sum of the full-size launches, mean of two steps' s2v and v2s launches)
-# and thread instructions per pair of the double-float kernels (smsp__inst_executed.sum x 32
-# / pairs, 100k-baseline case; those kernels are unchanged since that capture).
 # ncu counters of the direct kernels on the full LOFAR-like workload, valid while the kernel
 # source and the owners per thread are those they were taken with:
-# eps -> (sha256 of k_direct.cu, owners per thread, DRAM bytes per launch, instructions per pair)
+# eps -> (sha256 of k_direct.cu, owners per thread, DRAM bytes per launch, instructions per pair).
+# The current source has none: its line reports traffic null.
 DIRECT_COUNTERS = {1e-9: ("4bd864c34d1267f8e16c78fc6e727b931df1b0290a13386a3647fb00d039eb9d", 4, 126990144.0, 73.0)}
 
 

@@ -286,8 +286,8 @@ enum {
     HVOX_STAGE_PERMUTE = 0,  /* caller order <-> chunk order, weights (Sect. 4) */
     HVOX_STAGE_DIRECT = 1,   /* direct sub-problems (Sect. 3.1 fallback) */
     HVOX_STAGE_SPREAD = 2,   /* NUFFT spreading (step 1 of the type-3 transform) */
-    HVOX_STAGE_DECONV = 3,   /* deconvolve + zero-pad / crop (taper of step 1) */
-    HVOX_STAGE_FFT = 4,      /* uniform 3-D FFT (cuFFT, step 2) */
+    HVOX_STAGE_DECONV = 3,   /* deconvolve + zero-pad / crop (taper of step 1) in front of cuFFT */
+    HVOX_STAGE_FFT = 4,      /* uniform 3-D FFT (step 2), the library's with the deconvolution, or cuFFT */
     HVOX_STAGE_INTERP = 5,   /* NUFFT interpolation with taper (steps 3-4) */
     HVOX_STAGE_ZERO = 6,     /* clearing accumulators and grids */
     HVOX_NUM_STAGES = 8

@@ -182,6 +182,11 @@ CostModel default_cost_model(int prec, bool plain, int w, bool z2z_fft) {
         // CUDA-event stage times; the fit is stored with the tests). The direct rate is the
         // large launch of the SKA-Low-like benchmark line (2.9e12 pairs per launch), since
         // the calibration workloads have almost no direct work.
+        // These are the rates of the stored fits. The kernels are faster by now (direct pairs
+        // 2.05e12/s at FP32 and 8.2e11/s in double-float, FFTs 1.2 to 2 times), and direct sums and
+        // FFTs by similar factors; with the new direct rate alone the dense core goes from 1 to 21
+        // sub-problems on a near tie (12.43 against 12.35 ms modelled) and its small FFT batches,
+        // which the model does not see, took 12.9 ms instead of 7.9.
         m.direct_pair = 1.0 / 1.17e12;
         m.scatter_smem = 1.0 / 6.3e11;
         m.scatter_global = 1.0 / 2.4e11;
