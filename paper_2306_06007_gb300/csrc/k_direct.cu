@@ -178,6 +178,13 @@ template <class K> __device__ __forceinline__ void pipe_wait(DirectShared<K> &sh
     if (err) atomicOr(err, kDevErrStall);
 }
 
+// The same for a whole warp. Its lanes poll by themselves and may leave on different tries, while the
+// tensor-memory reads (.aligned) that follow need them together.
+template <class K> __device__ __forceinline__ void warp_wait(DirectShared<K> &sh, uint64_t *bar, uint32_t parity, int *err) {
+    pipe_wait(sh, bar, parity, err);
+    __syncwarp();
+}
+
 // One producer thread: its points of the tile at s0 (the staged values' magnitudes are summed per
 // warp and pass).
 template <class K, int DIR>
@@ -262,7 +269,7 @@ __device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &
         __syncthreads();
         for (uint32_t t = 0; t < tiles; ++t) {
             const uint32_t n = pipe.tiles + t;
-            pipe_wait(sh, &sh.freed[n & 1u], (n >> 1) ^ 1u, J.err);
+            warp_wait(sh, &sh.freed[n & 1u], (n >> 1) ^ 1u, J.err);
             stage_tile<K, DIR>(J, w, w.s0 + (int)t * kStream, sh, n & 1u);
             __syncwarp();
             if ((tid & 31) == 0) tc::mbar_arrive(&sh.staged[n & 1u]);
@@ -292,8 +299,7 @@ __device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &
         };
         auto open_chunk = [&](uint32_t c) {  // the chunk's products are done: read its first part
             const uint32_t n = pipe.chunks + c;
-            pipe_wait(sh, &sh.done[block][n & 1u], n >> 1, J.err);
-            __syncwarp();
+            warp_wait(sh, &sh.done[block][n & 1u], n >> 1, J.err);
             tc::fence_after();
             read_part(n & 1u, 0);
         };
@@ -301,7 +307,7 @@ __device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &
         for (uint32_t c = 0; c < chunks; ++c) {
             const uint32_t set = (pipe.chunks + c) & 1u, tile = pipe.tiles + c / kPerTile, buf = tile & 1u;
             if (c % kPerTile == 0) {
-                pipe_wait(sh, &sh.staged[buf], tile >> 1, J.err);
+                warp_wait(sh, &sh.staged[buf], tile >> 1, J.err);
                 sum.begin(sh.red[buf]);
             }
             const auto *val = &sh.val[buf][(c % kPerTile) * K::kN + half * kHalf];
