@@ -70,8 +70,10 @@ typedef enum {
     HVOX_ENOMEM = 2,        /* device or host allocation failed */
     HVOX_ECUDA = 3,         /* a CUDA runtime or cuFFT call failed */
     HVOX_ETIMEOUT = 4,      /* a direct-sum kernel's bounded wait inside its own pipeline (never on
-                               another kernel or a peer) ran out after ~2 s: reported like the
-                               device error word below; its outputs are NaN */
+                               another kernel or a peer) ran out after ~0.4 s: reported like the
+                               device error word below. Every output that misses terms is NaN,
+                               also those of other plans of the same batched call, which then
+                               report it too */
     HVOX_EUNSUPPORTED = 5,  /* option combination not supported */
     HVOX_EINTERNAL = 6      /* internal invariant violated; also the plan's device error
                                word: a kernel found a spreading or interpolation window
@@ -364,7 +366,8 @@ const char *hvox_version(void);
  * call before any stream capture. All calls share the array and it keeps the last call's
  * contents, so calls whose work overlaps on the GPU (different streams, or different
  * host threads) race: serialise them. The sum over pixels runs in segments whose partial
- * sums meet through atomic adds, so the last bits of V may differ between calls. Asynchronous on `stream`.
+ * sums meet through atomic adds, so the last bits of V may differ between calls. Asynchronous on `stream`:
+ * nothing reads a device error word afterwards, so a wait that ran out (HVOX_ETIMEOUT) shows as NaN in V only.
  */
 hvox_status hvox_direct_synthesize_noalloc(const double *pix_xyz, int64_t n_pix, const double *uvw, int64_t n_vis,
                                            const float *I, float *V, int isign, void *stream);

@@ -150,8 +150,9 @@ void run_waves(Plan &p, int dir, const In *src, Out *acc, cudaStream_t s, Profil
 DirectJob job_of_plan(const Plan &p, int dir) {
     const float4 *ph = p.pix_hi.as<float4>(), *pl = p.pix_lo.as<float4>();
     const float4 *vh = p.vis_hi.as<float4>(), *vl = p.vis_lo.as<float4>();
-    if (dir == 0) return {vh, vl, ph, pl, p.src.ptr, p.acc.ptr, (float)p.isign, p.pix_scale, p.vis_scale, p.err.as<int>()};
-    return {ph, pl, vh, vl, p.src.ptr, p.acc.ptr, (float)p.isign, p.pix_scale, p.vis_scale, p.err.as<int>()};
+    int *err = p.err.as<int>();
+    if (dir == 0) return {vh, vl, ph, pl, p.src.ptr, p.acc.ptr, (float)p.isign, p.pix_scale, p.vis_scale, err, p.stall};
+    return {ph, pl, vh, vl, p.src.ptr, p.acc.ptr, (float)p.isign, p.pix_scale, p.vis_scale, err, p.stall};
 }
 
 // The direct sums of one plan in a launch of their own.

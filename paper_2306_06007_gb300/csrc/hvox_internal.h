@@ -40,7 +40,10 @@ void check_cufft(cufftResult r, const char *what);
 //   capture  a CUDA-graph capture (the plan falls back to eager launches);
 //   window   the pixel scale of the NUFFT sub-problem with the most pixels is multiplied
 //            by 4 on the host, so its kernels clamp the pixels' windows into the grid and
-//            set the device error word (hvox_sync then returns HVOX_EINTERNAL).
+//            set the device error word (hvox_sync then returns HVOX_EINTERNAL);
+//   stall    the direct kernels of a plan (or of a call that allocates nothing) never hand a
+//            staged tile on, so that their bounded waits run out and they report
+//            HVOX_ETIMEOUT (nothing is in flight on the tensor cores then).
 // No GPU fault is involved: every injected failure is raised or prepared on the host.
 bool fault_hit(const char *site);
 
@@ -117,7 +120,8 @@ struct DirectJob {
     void *acc;
     float sgn;
     float pix_scale, vis_scale;
-    int *err;  // the plan's device error word (may be null)
+    int *err;   // the plan's device error word (may be null)
+    int stall;  // tiles are never handed on, so that the waits run out (fault_hit "stall")
 };
 
 // The two powers of two for pixels of largest |coordinate| top (1 for unit vectors).
@@ -421,6 +425,7 @@ struct Plan {
     int ntrans = 1;
     int direct_kind = 0;           // kDirectF32, ...
     float pix_scale = 1.f, vis_scale = 1.f;  // coord_scales of the pixels
+    bool stall = false;            // DirectJob::stall of its launches
     double sigma = 2.0;
     double budget_opt = 0.0;       // chunk_budget_bytes option (0 -> cost-model search)
     bool sigma_auto = true;        // upsampling chosen by the planner

@@ -162,6 +162,7 @@ template <class K> struct __align__(128) DirectShared {
     uint64_t done[2][2];                       // [row block][set]: a chunk's products have finished
     uint64_t read[2][2];                       // [row block][set]: its eight warps have read the set
     uint64_t staged[2], freed[2];              // [buffer]: tile written / tile summed by every consumer
+    uint64_t drained;                          // after a wait ran out: every product issued has finished
     uint32_t tmem;
     int next, abort;
 };
@@ -172,10 +173,18 @@ struct DirectPipe {
     uint32_t tmem, chunks, tiles;
 };
 
-template <class K> __device__ __forceinline__ void pipe_wait(DirectShared<K> &sh, uint64_t *bar, uint32_t parity, int *err) {
-    if (*(volatile int *)&sh.abort || tc::mbar_wait(bar, parity & 1u)) return;
-    *(volatile int *)&sh.abort = 1;  // later waits are skipped and the CTA ends after this item
+// A bounded wait: false where it ran out, here or in another thread of the CTA. Then nothing waits any
+// longer, no more products are issued, the item's sums become NaN and so do those of every item that
+// the CTA takes after it (an item left out would be missing from a finite result); the products
+// in flight are waited for before tensor memory is given back (direct_end).
+template <class K> __device__ __forceinline__ bool pipe_wait(DirectShared<K> &sh, uint64_t *bar, uint32_t parity, int *err) {
+    for (int i = 0; i < tc::kWaitLimit; ++i) {
+        if (*(volatile int *)&sh.abort) return false;
+        if (tc::mbar_try(bar, parity & 1u)) return true;
+    }
+    *(volatile int *)&sh.abort = 1;
     if (err) atomicOr(err, kDevErrStall);
+    return false;
 }
 
 // The same for a whole warp. Its lanes poll by themselves and may leave on different tries, while the
@@ -234,11 +243,11 @@ __device__ __forceinline__ void issue_chunks(DirectShared<K> &sh, const DirectPi
     const uint64_t dig0 = tc::operand_desc(tc::smem_addr(sh.dig), sizeof(sh.dig[0][0]));
     for (uint32_t c = 0; c < chunks; ++c) {
         const uint32_t n = pipe.chunks + c, set = n & 1u, tile = pipe.tiles + c / kPerTile;
-        if (c % kPerTile == 0) pipe_wait(sh, &sh.staged[tile & 1u], tile >> 1, err);
+        if (c % kPerTile == 0 && !pipe_wait(sh, &sh.staged[tile & 1u], tile >> 1, err)) return;
         const uint64_t dig = dig0 + (((tile & 1u) * sizeof(sh.dig[0]) + (c % kPerTile) * K::kN * 16) >> 4);
 #pragma unroll
         for (int block = 0; block < 2; ++block) {
-            pipe_wait(sh, &sh.read[block][set], (n >> 1) ^ 1u, err);
+            if (!pipe_wait(sh, &sh.read[block][set], (n >> 1) ^ 1u, err)) return;
             tc::fence_after();
             const uint32_t d = pipe.tmem + set_columns<K>(block, set);
 #pragma unroll
@@ -251,8 +260,9 @@ __device__ __forceinline__ void issue_chunks(DirectShared<K> &sh, const DirectPi
     }
 }
 
+// Sums one item; whether a wait ran out (the same in every thread).
 template <class K, int DIR>
-__device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &w, DirectShared<K> &sh, DirectPipe &pipe) {
+__device__ __forceinline__ bool direct_item(const DirectJob &J, const WorkItem &w, DirectShared<K> &sh, DirectPipe &pipe) {
     using Form = typename K::Form;
     using Side = std::conditional_t<DIR == 0, typename Form::P, typename Form::R>;
     constexpr uint32_t kPerTile = kStream / K::kN;
@@ -272,7 +282,7 @@ __device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &
             warp_wait(sh, &sh.freed[n & 1u], (n >> 1) ^ 1u, J.err);
             stage_tile<K, DIR>(J, w, w.s0 + (int)t * kStream, sh, n & 1u);
             __syncwarp();
-            if ((tid & 31) == 0) tc::mbar_arrive(&sh.staged[n & 1u]);
+            if ((tid & 31) == 0 && !J.stall) tc::mbar_arrive(&sh.staged[n & 1u]);
         }
     } else {
         const int block = tid >> 8, half = (tid >> 7) & 1, row = block * 128 + (tid & 127);
@@ -336,6 +346,19 @@ __device__ __forceinline__ void direct_item(const DirectJob &J, const WorkItem &
     }
     pipe.chunks += chunks;
     pipe.tiles += tiles;
+    return __syncthreads_or(*(volatile int *)&sh.abort) != 0;
+}
+
+// An item that a CTA takes after one of its waits ran out.
+template <class K> __device__ __forceinline__ void poison_item(const DirectJob &J, const WorkItem &w) {
+    const int k = w.o0 + (int)threadIdx.x;
+    if ((int)threadIdx.x < kRows && k < w.o1) {
+        typename K::Sum sum;
+        sum.clear();
+        sum.poison();
+        sum.store(J, k);
+    }
+    if (threadIdx.x == 0 && J.err) atomicOr(J.err, kDevErrStall);
 }
 
 template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShared<K> &sh) {
@@ -350,6 +373,7 @@ template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShar
             tc::mbar_init(&sh.staged[i], kProducers / 32);
             tc::mbar_init(&sh.freed[i], kConsumers / 32);
         }
+        tc::mbar_init(&sh.drained, 1);
         sh.abort = 0;
     }
     tc::fence_before();
@@ -358,7 +382,13 @@ template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShar
     return {sh.tmem, 0u, 0u};
 }
 
-template <class K> __device__ __forceinline__ void direct_end(DirectShared<K> &sh, const DirectPipe &pipe) {
+template <class K> __device__ __forceinline__ void direct_end(DirectShared<K> &sh, const DirectPipe &pipe, bool stopped) {
+    // Without the consumers' waits, products may still be reading shared memory and writing tensor memory.
+    if (stopped && threadIdx.x == kIssuer) {
+        tc::mma_commit(&sh.drained);
+        for (int i = 0; i < tc::kWaitLimit && !tc::mbar_try(&sh.drained, 0u); ++i) {}
+    }
+    __syncwarp();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -580,9 +610,15 @@ __global__ void __launch_bounds__(kDirectThreads, 1)
             const float4 e = gT[2 * (i / kDfCopies)];
             sh.extra.e[i] = make_float4(e.x, e.z, e.y, e.w);
         }
-    for (int it = blockIdx.x; it < n_items && !sh.abort; it = next_item(counter, sh.next))
-        direct_item<K, DIR>(job_of<BATCH>(J0, jobs, item_job, it), items[it], sh, pipe);
-    direct_end(sh, pipe);
+    bool stopped = false;
+    for (int it = blockIdx.x; it < n_items; it = next_item(counter, sh.next)) {
+        const DirectJob J = job_of<BATCH>(J0, jobs, item_job, it);
+        if (stopped)
+            poison_item<K>(J, items[it]);
+        else
+            stopped = direct_item<K, DIR>(J, items[it], sh, pipe);
+    }
+    direct_end(sh, pipe, stopped);
 }
 
 // ------------------------------------------------------------- FP64
@@ -875,12 +911,16 @@ __device__ __forceinline__ void noalloc_items(const DirectJob &J, int n_vis, int
             for (int c = 0; c < kDfCopies; ++c) sh.extra.e[i * kDfCopies + c] = e;
         }
     const int tiles = (n_vis + kRows - 1) / kRows, items = tiles * ((n_pix + seg - 1) / seg);
-    for (int it = blockIdx.x; it < items && !sh.abort; it += gridDim.x) {
+    bool stopped = false;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {  // direct_item ends in a barrier
         const int o0 = it % tiles * kRows, s0 = it / tiles * seg;
-        direct_item<K, 0>(J, WorkItem{o0, min(o0 + kRows, n_vis), s0, min(s0 + seg, n_pix)}, sh, pipe);
-        __syncthreads();  // the owners' digits have had their last reader
+        const WorkItem w{o0, min(o0 + kRows, n_vis), s0, min(s0 + seg, n_pix)};
+        if (stopped)
+            poison_item<K>(J, w);
+        else
+            stopped = direct_item<K, 0>(J, w, sh, pipe);
     }
-    direct_end(sh, pipe);
+    direct_end(sh, pipe, stopped);
 }
 
 __global__ void __launch_bounds__(kDirectThreads, 1)
@@ -948,7 +988,7 @@ extern "C" hvox_status hvox_direct_synthesize_noalloc(const double *pix_xyz, int
         check_cuda(cudaGetLastError(), "noalloc_prepare");
         const int64_t tiles = (n_vis + kRows - 1) / kRows;
         const int64_t seg = direct_segment(tiles, n_pix), items = tiles * ((n_pix + seg - 1) / seg);
-        const DirectJob J{vh, vl, rh, rl, I, V, (float)isign, 1.f, 1.f, nullptr};
+        const DirectJob J{vh, vl, rh, rl, I, V, (float)isign, 1.f, 1.f, nullptr, fault_hit("stall")};
         constexpr size_t smem = sizeof(DirectShared<DfKind<0, float>>);
         static_assert(smem >= sizeof(DirectShared<F32Kind<0>>), "either form");
         allow_smem<DirectJob>(direct_noalloc_kernel, smem);

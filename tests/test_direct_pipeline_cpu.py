@@ -21,7 +21,16 @@ def test_warps_meet_before_aligned_instructions():
     # tcgen05.ld and tcgen05.wait::ld are .aligned: every wait of the warps that use them is a whole
     # warp's, and only the issuing thread waits by itself.
     src = open(os.path.join(CSRC, "k_direct.cu")).read()
-    item = _body(src, "void direct_item")
+    item = _body(src, " direct_item")
     assert "tmem_load_wait" in item and len(re.findall(r"\bwarp_wait\(", item)) >= 3
     assert not re.search(r"\bpipe_wait\(|\bmbar_wait\(", item), "a per-thread wait in front of aligned instructions"
     assert re.search(r"pipe_wait\(.*?\);\s*__syncwarp\(\);\s*}$", _body(src, "void warp_wait"), re.S)
+
+
+def test_products_end_before_tensor_memory_is_freed():
+    # A wait that ran out stops the issuing thread, and what it had issued is waited for (with a
+    # limit) before the CTA gives its memory back.
+    src = open(os.path.join(CSRC, "k_direct.cu")).read()
+    issue, end = _body(src, "void issue_chunks"), _body(src, "void direct_end")
+    assert len(re.findall(r"if \([^;]*!pipe_wait\(.*\)\) return;", issue)) == len(re.findall(r"pipe_wait\(", issue)) == 2
+    assert end.index("mma_commit(&sh.drained)") < end.index("mbar_try(&sh.drained") < end.index("tmem_free")
