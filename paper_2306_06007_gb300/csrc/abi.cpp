@@ -44,6 +44,12 @@ void check_cufft(cufftResult r, const char *what) {
     }
 }
 
+int current_device() {
+    int dev = 0;
+    check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+    return dev;
+}
+
 bool fault_hit(const char *site) {
     static std::mutex mu;
     static std::string spec;

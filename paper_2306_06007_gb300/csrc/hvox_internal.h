@@ -13,6 +13,8 @@
 #include <tuple>
 #include <vector>
 
+#include "per_device.h"
+
 #include "../../include/hvox.h"
 
 namespace hvox {
@@ -31,6 +33,7 @@ struct Error {
 [[noreturn]] void fail(hvox_status code, const std::string &msg);
 void check_cuda(cudaError_t e, const char *what);
 void check_cufft(cufftResult r, const char *what);
+int current_device();
 
 // Host-side fault injection for tests. HVOX_FAULT = "site:n[,site:n...]" makes the n-th
 // event of each named site (counted from the moment the variable last changed) fail the

@@ -33,7 +33,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <mutex>
 #include <type_traits>
 
 #include "hvox_internal.h"
@@ -490,8 +489,8 @@ int rows_per_cta(const CfftDev &d) {
 }
 
 void set_attrs() {
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static OncePerDevice once;
+    once.run(current_device(), [] {
         auto allow = [](auto k, int bytes) {
             check_cuda(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes), "cudaFuncSetAttribute");
         };

@@ -22,7 +22,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <mutex>
 
 #include "dfloat.cuh"
 #include "hvox_internal.h"
@@ -348,8 +347,8 @@ template <int SG> void allow_sign() {
 }
 
 void set_fft_attrs() {
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static OncePerDevice once;
+    once.run(current_device(), [] {
         allow_sign<1>();
         allow_sign<-1>();
     });

@@ -750,14 +750,13 @@ int direct_tile(int kind) { return kind == kDirectF64 ? kTile : kRows; }
 int direct_owners_per_thread(int kind) { return kind == kDirectF64 ? kPerThread : 1; }
 
 static int sm_count() {
-    static std::atomic<int> sms{0};
-    int n = sms.load();
+    static std::atomic<int> sms[256];
+    const int dev = current_device();
+    int n = dev < 256 ? sms[dev].load() : 0;
     if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         if (n <= 0) n = 152;
-        sms.store(n);
+        if (dev < 256) sms[dev].store(n);
     }
     return n;
 }
@@ -767,15 +766,13 @@ static unsigned grid_for(int64_t n_items, int per_sm) {
     return (unsigned)std::max<int64_t>(1, std::min<int64_t>(n_items, (int64_t)sm_count() * per_sm));
 }
 
-// Dynamic shared memory of a kernel, allowed once per device (Once names the kernel).
-template <class Once, class F> static void allow_smem(F kernel, size_t bytes) {
-    static std::atomic<uint64_t> done[4];
-    int dev = 0;
-    check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
-    if (dev < 256 && (done[dev / 64].load() >> (dev % 64) & 1)) return;
-    check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
-               "cudaFuncSetAttribute");
-    if (dev < 256) done[dev / 64].fetch_or(uint64_t(1) << (dev % 64));
+// Dynamic shared memory of a kernel (Kernel names it).
+template <class Kernel, class F> static void allow_smem(F kernel, size_t bytes) {
+    static OncePerDevice once;
+    once.run(current_device(), [&] {
+        check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes),
+                   "cudaFuncSetAttribute");
+    });
 }
 
 template <class K, int DIR, bool BATCH> struct DirectOnce {};

@@ -27,7 +27,6 @@
 #include <algorithm>
 #include <climits>
 #include <cstdint>
-#include <mutex>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -1445,9 +1444,8 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 
 // Dynamic shared memory of the spreading kernels: the tile (real and imaginary planes).
 template <typename T, int W> void set_smem_attrs() {
-    // Once per instantiation, also when plans are built and run on several host threads.
-    static std::once_flag once;
-    std::call_once(once, [] {
+    static OncePerDevice once;
+    once.run(current_device(), [] {
         for (auto k : {spread_pix_kernel<T, W, false>, spread_pix_kernel<T, W, sizeof(T) == 8>})
             check_cuda(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_bytes<T, W>()),
                        "cudaFuncSetAttribute");
