@@ -7,8 +7,8 @@
 // The phase <p, r> reaches ~1e5 turns, so it is never formed in plain FP32. Every
 // coordinate is stored as a pair of floats hi + lo (hi = fl32(x), lo = fl32(x - hi)), and the
 // tensor cores form the turns modulo one of a tile of pairs from their digits (phase_tc.cuh):
-//  * FP32 path (eps >= 1e-6): fraction in FP32 (error ~1.5e-8 turn rms), hardware sin/cos
-//    approximations, FP32 accumulation;
+//  * FP32 path (eps >= 1e-6): fraction in FP32 (error ~5e-9 turn rms up to 2^22 turns, 1e-7 at 2^28),
+//    hardware sin/cos approximations, FP32 accumulation;
 //  * double-float path (eps < 1e-6): exp(j 2 pi f) as the hi parts of a 1024-entry table of
 //    exp(j 2 pi m / 1024) plus a lo part (the table's lo parts and a short series in the
 //    remainder, in plain float; error ~1e-10); sums in double-float arithmetic (Dekker 1971);
