@@ -460,7 +460,7 @@ void build_plan(Plan &p, const double *pix_in, const double *uvw_in, const doubl
         for (double v : uvw) far = std::max(far, std::fabs((float)v));
         far *= p.vis_scale;
         if (p.direct_kind == kDirectF32 && !(far <= kF32Reach)) p.direct_kind = kDirectWide;
-        if (p.direct_kind == kDirectDf && !(far <= kDfReach)) p.direct_kind = kDirectF64;
+        if (!(far <= kDfReach)) p.direct_kind = kDirectF64;
         p.stall = fault_hit("stall");
         std::vector<WorkItem> a, b;
         build_items(part.rects, true, p.direct_kind, a);

@@ -163,12 +163,9 @@ void run_direct(Plan &p, int dir, cudaStream_t s) {
     check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset item counter");
     if (p.direct_kind != kDirectF64)
         launch_direct(p.direct_kind, dir, it, n, counter, job_of_plan(p, dir), p.cis_tab.as<float4>(), s);
-    else if (dir == 0)
-        launch_direct_s2v_f64(it, n, counter, p.vis_xyz.as<double>(), p.n_vis, p.pix_xyz.as<double>(), p.n_pix,
-                              p.src.as<double>(), p.acc.as<double2>(), p.isign, s);
     else
-        launch_direct_v2s_f64(it, n, counter, p.pix_xyz.as<double>(), p.n_pix, p.vis_xyz.as<double>(), p.n_vis,
-                              p.src.as<double2>(), p.acc.as<double>(), p.isign, s);
+        launch_direct_f64(p.prec, dir, it, n, counter, p.vis_xyz.as<double>(), p.n_vis, p.pix_xyz.as<double>(), p.n_pix,
+                          p.src.ptr, p.acc.ptr, p.isign, s);
 }
 
 // sky -> vis between the permutations: src (chunk-ordered c_n) -> acc (chunk-ordered V).

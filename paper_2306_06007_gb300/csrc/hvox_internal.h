@@ -141,8 +141,8 @@ __host__ __device__ inline void coord_scales(float top, float &pix_scale, float 
 enum { kDirectF32 = 0, kDirectDf = 1, kDirectF64 = 2, kDirectWide = 3 };
 
 // Largest |p_d| times pixel scale (turns per dimension) that the digits of each form reach: an
-// FP32 plan beyond its reach runs the double-float form on its float values, a double-float
-// one the FP64 kernels.
+// FP32 plan beyond its reach runs the double-float form on its float values, and beyond the
+// double-float reach either runs the FP64 kernels.
 constexpr float kF32Reach = 0x1p28f, kDfReach = 0x1p33f;
 
 // Streamed points per work item for a rectangle of `tiles` owner tiles x `n` streamed points,
@@ -513,10 +513,8 @@ void launch_direct(int kind, int dir, const WorkItem *items, int64_t n, int *cou
                    const float4 *tab, cudaStream_t s);
 void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob *jobs,
                          const int *item_job, const float4 *tab, cudaStream_t s);
-void launch_direct_s2v_f64(const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
-                           const double *pxyz, int64_t np, const double *c, double2 *acc, int isign, cudaStream_t s);
-void launch_direct_v2s_f64(const WorkItem *items, int64_t n, int *counter, const double *pxyz, int64_t np,
-                           const double *vxyz, int64_t nv, const double2 *V, double *acc, int isign, cudaStream_t s);
+void launch_direct_f64(int prec, int dir, const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
+                       const double *pxyz, int64_t np, const void *src, void *acc, int isign, cudaStream_t s);
 
 // NUFFT sub-problems, one wave at a time (k_nufft.cu). g1 / g2: the lane's grid buffers.
 template <typename T>

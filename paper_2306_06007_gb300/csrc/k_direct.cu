@@ -14,8 +14,8 @@
 //    remainder, in plain float; error ~1e-10); sums in double-float arithmetic (Dekker 1971);
 //  * wide path: the double-float path on the values of an FP32 plan whose |p_d r_d| exceed 2^28
 //    turns (the reach of the FP32 digits);
-//  * plain path: everything in FP64 (the reference form the optimised paths replace; also for
-//    |p_d r_d| above 2^33 turns).
+//  * plain path: everything in FP64 (the reference form the optimised paths replace; also, on the
+//    plan's own values, for |p_d r_d| above 2^33 turns, the reach of the double-float digits).
 //
 // What bounds them: at FP32 the sine unit (two results a pair at 8 cycles for 32: 16 cycles of
 // the 20 that 32 pairs take), in double-float the FMA pipe (60% busy), the shared-memory pipe (63%)
@@ -623,12 +623,14 @@ __global__ void __launch_bounds__(kDirectThreads, 1)
 
 // ------------------------------------------------------------- FP64
 
-// Plain FP64 reference form.
-template <int VPT>
+template <class T> using cplx_of = std::conditional_t<sizeof(T) == 4, float2, double2>;
+
+// Plain FP64 reference form (T: the plan's real type).
+template <class T, int VPT>
 __global__ void __launch_bounds__(kThreads) direct_s2v_f64(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter,
                                                            const double *__restrict__ vxyz, int64_t nv_all,
                                                            const double *__restrict__ pxyz, int64_t np_all,
-                                                           const double *__restrict__ c, double2 *__restrict__ acc,
+                                                           const T *__restrict__ c, cplx_of<T> *__restrict__ acc,
                                                            double sgn) {
     __shared__ double sx[kThreads], sy[kThreads], sz[kThreads], sw[kThreads];
     __shared__ int s_next;
@@ -651,7 +653,7 @@ __global__ void __launch_bounds__(kThreads) direct_s2v_f64(const WorkItem *__res
             sx[threadIdx.x] = ok ? pxyz[n] : 0.0;
             sy[threadIdx.x] = ok ? pxyz[np_all + n] : 0.0;
             sz[threadIdx.x] = ok ? pxyz[2 * np_all + n] : 0.0;
-            sw[threadIdx.x] = ok ? c[n] : 0.0;
+            sw[threadIdx.x] = ok ? (double)c[n] : 0.0;
             __syncthreads();
             const int cnt = min(kThreads, w.s1 - s0);
             for (int q = 0; q < cnt; ++q) {
@@ -670,18 +672,18 @@ __global__ void __launch_bounds__(kThreads) direct_s2v_f64(const WorkItem *__res
         for (int v = 0; v < VPT; ++v) {
             int k = w.o0 + threadIdx.x + v * kThreads;
             if (k < w.o1) {
-                atomicAdd(&acc[k].x, are[v]);
-                atomicAdd(&acc[k].y, sgn * aim[v]);
+                atomicAdd(&acc[k].x, (T)are[v]);
+                atomicAdd(&acc[k].y, (T)(sgn * aim[v]));
             }
         }
     }
 }
 
-template <int VPT>
+template <class T, int VPT>
 __global__ void __launch_bounds__(kThreads) direct_v2s_f64(const WorkItem *__restrict__ items, int n_items, int *__restrict__ counter,
                                                            const double *__restrict__ pxyz, int64_t np_all,
                                                            const double *__restrict__ vxyz, int64_t nv_all,
-                                                           const double2 *__restrict__ V, double *__restrict__ acc,
+                                                           const cplx_of<T> *__restrict__ V, T *__restrict__ acc,
                                                            double sgn) {
     __shared__ double sx[kThreads], sy[kThreads], sz[kThreads], sr[kThreads], si[kThreads];
     __shared__ int s_next;
@@ -704,9 +706,8 @@ __global__ void __launch_bounds__(kThreads) direct_v2s_f64(const WorkItem *__res
             sx[threadIdx.x] = ok ? vxyz[k] : 0.0;
             sy[threadIdx.x] = ok ? vxyz[nv_all + k] : 0.0;
             sz[threadIdx.x] = ok ? vxyz[2 * nv_all + k] : 0.0;
-            double2 val = ok ? V[k] : make_double2(0.0, 0.0);
-            sr[threadIdx.x] = val.x;
-            si[threadIdx.x] = sgn * val.y;
+            sr[threadIdx.x] = ok ? (double)V[k].x : 0.0;
+            si[threadIdx.x] = ok ? sgn * (double)V[k].y : 0.0;
             __syncthreads();
             const int cnt = min(kThreads, w.s1 - s0);
             for (int q = 0; q < cnt; ++q) {
@@ -723,7 +724,7 @@ __global__ void __launch_bounds__(kThreads) direct_v2s_f64(const WorkItem *__res
 #pragma unroll
         for (int v = 0; v < VPT; ++v) {
             int n = w.o0 + threadIdx.x + v * kThreads;
-            if (n < w.o1) atomicAdd(&acc[n], a[v]);
+            if (n < w.o1) atomicAdd(&acc[n], (T)a[v]);
         }
     }
 }
@@ -822,20 +823,23 @@ void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, in
     if (n > 0) launch_kind<true>(kind, dir, items, n, counter, DirectJob{}, jobs, item_job, tab, s);
 }
 
-void launch_direct_s2v_f64(const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
-                           const double *pxyz, int64_t np, const double *c, double2 *acc, int isign, cudaStream_t s) {
-    if (n <= 0) return;
-    direct_s2v_f64<kPerThread><<<grid_for(n, 4), kThreads, 0, s>>>(items, (int)n, counter, vxyz, nv, pxyz, np, c, acc,
-                                                                   (double)isign);
-    check_cuda(cudaGetLastError(), "direct_s2v_f64");
+template <class T>
+static void launch_f64(int dir, const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
+                       const double *pxyz, int64_t np, const void *src, void *acc, double sgn, cudaStream_t s) {
+    if (dir == 0)
+        direct_s2v_f64<T, kPerThread><<<grid_for(n, 4), kThreads, 0, s>>>(
+            items, (int)n, counter, vxyz, nv, pxyz, np, static_cast<const T *>(src), static_cast<cplx_of<T> *>(acc), sgn);
+    else
+        direct_v2s_f64<T, kPerThread><<<grid_for(n, 4), kThreads, 0, s>>>(
+            items, (int)n, counter, pxyz, np, vxyz, nv, static_cast<const cplx_of<T> *>(src), static_cast<T *>(acc), sgn);
+    check_cuda(cudaGetLastError(), "direct sums (FP64)");
 }
 
-void launch_direct_v2s_f64(const WorkItem *items, int64_t n, int *counter, const double *pxyz, int64_t np,
-                           const double *vxyz, int64_t nv, const double2 *V, double *acc, int isign, cudaStream_t s) {
+void launch_direct_f64(int prec, int dir, const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
+                       const double *pxyz, int64_t np, const void *src, void *acc, int isign, cudaStream_t s) {
     if (n <= 0) return;
-    direct_v2s_f64<kPerThread><<<grid_for(n, 4), kThreads, 0, s>>>(items, (int)n, counter, pxyz, np, vxyz, nv, V, acc,
-                                                                   (double)isign);
-    check_cuda(cudaGetLastError(), "direct_v2s_f64");
+    const auto launch = prec == 1 ? launch_f64<float> : launch_f64<double>;
+    launch(dir, items, n, counter, vxyz, nv, pxyz, np, src, acc, (double)isign, s);
 }
 
 }  // namespace hvox
@@ -892,7 +896,7 @@ __global__ void noalloc_prepare_kernel(const double *__restrict__ pix, int64_t n
     if ((threadIdx.x & 31) == 0 && mv != 0u) atomicMax(top + 1, mv);
 }
 
-// The FP32 direct sums (the wide form beyond the FP32 digits' reach) over items in a fixed order
+// The FP32 direct sums (beyond the FP32 digits' reach the wide form, beyond that FP64) over items in a fixed order
 // instead of a work list; the segments' sums meet in V through atomicAdd, so their order (and
 // the last bits of the result) is not deterministic.
 template <class K>
@@ -920,14 +924,43 @@ __device__ __forceinline__ void noalloc_items(const DirectJob &J, int n_vis, int
     direct_end(sh, pipe, stopped);
 }
 
+// The same in FP64, an owner to a thread: correct where the digits end, and not tuned (no instrument has 2^33
+// turns).
+__device__ __noinline__ void noalloc_items_f64(const double *__restrict__ pix, const double *__restrict__ uvw,
+                                               const float *__restrict__ c, float2 *__restrict__ acc, double sgn,
+                                               int n_vis, int n_pix, int seg) {
+    const int tiles = (n_vis + kRows - 1) / kRows, items = tiles * ((n_pix + seg - 1) / seg);
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        const int k = it % tiles * kRows + (int)threadIdx.x, s0 = it / tiles * seg;
+        if ((int)threadIdx.x >= kRows || k >= n_vis) continue;
+        double re = 0.0, im = 0.0;
+        for (int n = s0; n < min(s0 + seg, n_pix); ++n) {
+            double t = fma(uvw[3 * (int64_t)k], pix[3 * (int64_t)n],
+                           fma(uvw[3 * (int64_t)k + 1], pix[3 * (int64_t)n + 1], uvw[3 * (int64_t)k + 2] * pix[3 * (int64_t)n + 2]));
+            t -= rint(t);
+            double sn, cs;
+            sincospi(2.0 * t, &sn, &cs);
+            re = fma((double)c[n], cs, re);
+            im = fma((double)c[n], sn, im);
+        }
+        atomicAdd(&acc[k].x, (float)re);
+        atomicAdd(&acc[k].y, (float)(sgn * im));
+    }
+}
+
 __global__ void __launch_bounds__(kDirectThreads, 1)
-    direct_noalloc_kernel(DirectJob J, int n_vis, int n_pix, int seg, const unsigned *__restrict__ top) {
+    direct_noalloc_kernel(DirectJob J, int n_vis, int n_pix, int seg, const unsigned *__restrict__ top,
+                          const double *__restrict__ pix, const double *__restrict__ uvw) {
     extern __shared__ __align__(128) unsigned char direct_smem[];
     coord_scales(__uint_as_float(top[0]), J.pix_scale, J.vis_scale);
-    if (__uint_as_float(top[1]) * J.vis_scale <= kF32Reach)
+    const float far = __uint_as_float(top[1]) * J.vis_scale;
+    if (far <= kF32Reach)
         noalloc_items<F32Kind<0>>(J, n_vis, n_pix, seg, direct_smem);
-    else
+    else if (far <= kDfReach)
         noalloc_items<DfKind<0, float>>(J, n_vis, n_pix, seg, direct_smem);
+    else
+        noalloc_items_f64(pix, uvw, static_cast<const float *>(J.val), static_cast<float2 *>(J.acc), (double)J.sgn, n_vis,
+                          n_pix, seg);
 }
 
 std::mutex g_noalloc_mu;
@@ -989,7 +1022,8 @@ extern "C" hvox_status hvox_direct_synthesize_noalloc(const double *pix_xyz, int
         constexpr size_t smem = sizeof(DirectShared<DfKind<0, float>>);
         static_assert(smem >= sizeof(DirectShared<F32Kind<0>>), "either form");
         allow_smem<DirectJob>(direct_noalloc_kernel, smem);
-        direct_noalloc_kernel<<<grid_for(items, 1), kDirectThreads, smem, s>>>(J, (int)n_vis, (int)n_pix, (int)seg, top);
+        direct_noalloc_kernel<<<grid_for(items, 1), kDirectThreads, smem, s>>>(J, (int)n_vis, (int)n_pix, (int)seg, top,
+                                                                                     pix_xyz, uvw);
         check_cuda(cudaGetLastError(), "direct_noalloc");
         set_error("");
         return HVOX_OK;
