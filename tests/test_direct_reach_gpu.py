@@ -48,10 +48,12 @@ def test_fp32_digits_hold_over_their_reach(gpu_lib, log2, scale):
 
 
 # Past the double-float digits (2^33 turns; their leading one is inexact in fp16 from 2^34 and infinite from
-# 2^39) the sums run in FP64, as the oracle's: a product of t turns rounds at 2^-53 t in each.
+# 2^39) the sums run in FP64, as the oracle's: a product of t turns rounds at 2^-53 t in each. Baselines within
+# 2e3 wavelengths of a far point: the host sizes grids by extents, slowly where these are 2^36.
 @pytest.mark.parametrize("log2", [33.5, 36, 40])
 def test_sums_beyond_every_digit(gpu_lib, log2):
-    radius = 2.0 ** log2
-    e = _errors(gpu_lib, 1e-4, *_points(400, 900, radius))
+    pix, uvw, sky, vis = _points(400, 900, 1e3)
+    uvw += 2.0 ** log2 * np.array([1.0, -1.0, 1.0])
+    e = _errors(gpu_lib, 1e-4, pix, uvw, sky, vis)
     print(f"2^{log2}: {e}")
-    assert max(e) <= 1e-6 + 2.0 * math.pi * 3.0 * radius * 2.0 ** -52
+    assert max(e) <= 1e-6 + 2.0 * math.pi * 3.0 * 2.0 ** log2 * 2.0 ** -52
