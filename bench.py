@@ -46,24 +46,6 @@ WORKLOAD = ("LOFAR-like: HEALPix nside=256 30deg cap (52,812 px) x 300 antennas 
 FP32_PEAK_FLOPS = 152 * 128 * 2 * 2.07e9  # FP32 FMA pipes x 2 flops x max SM clock
 FLOPS_PER_PAIR = 16.0                      # algorithmic flops per (pixel, baseline) pair
 
-# ncu counters of the direct kernels on the full LOFAR-like workload, valid while the kernel
-# source and the owners per thread are those they were taken with:
-# eps -> (sha256 of k_direct.cu, owners per thread, DRAM bytes per launch, instructions per pair).
-# The current source has none: its line reports traffic null.
-DIRECT_COUNTERS = {1e-9: ("4bd864c34d1267f8e16c78fc6e727b931df1b0290a13386a3647fb00d039eb9d", 4, 126990144.0, 73.0)}
-
-
-def direct_counters(eps, config, other_workload, n_vis, vpt):
-    """(traffic bytes per launch, instructions per pair) or (None, None)."""
-    import hashlib
-    entry = DIRECT_COUNTERS.get(eps)
-    if entry is None or config != 2 or other_workload or n_vis or vpt != entry[1]:
-        return None, None
-    path = os.path.join(ROOT, "paper_2306_06007_gb300", "csrc", "k_direct.cu")
-    with open(path, "rb") as f:
-        digest = hashlib.sha256(f.read()).hexdigest()
-    return (entry[2], entry[3]) if digest == entry[0] else (None, None)
-
 
 def dist_env():
     return int(os.environ.get("RANK", "0")), int(os.environ.get("WORLD_SIZE", "1")), int(os.environ.get("LOCAL_RANK", "0"))
@@ -463,21 +445,14 @@ def run_gpu(args):
     if dom == "direct":
         pairs_per_launch = info["direct_pairs"]
         achieved = pairs_per_launch * FLOPS_PER_PAIR / avg_s
-        traffic, ipp = direct_counters(args.eps, args.config, args.core_radius or args.radius_km, args.n_vis,
-                                       info.get("direct_vpt"))
         roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": FP32_PEAK_FLOPS / 1e12,
-                    "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_FLOPS, "traffic": traffic,
-                    "kernel": "direct_s2v + direct_v2s (one launch each per step)",
+                    "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_FLOPS, "traffic": None,
+                    "kernel": "direct_kernel (one launch per direction and step)",
                     "pairs_per_launch": pairs_per_launch, "avg_launch_ms": avg_s * 1e3,
                     "pairs_per_s": pairs_per_launch / avg_s,
                     "peak_note": "FP32 pipes 152 SMs x 128 lanes x 2 flops x 2.07 GHz (derived)"}
         if peaks:
             roofline["frac_of_probe"] = achieved / peaks["fp32_flops"]
-        if ipp is not None:
-            # FP32-pipe instruction issue against the same pipes' peak (one instruction per
-            # lane per cycle): how close the kernel runs to the hardware it is bound by.
-            roofline["instr_per_pair"] = ipp
-            roofline["issue_frac"] = ipp * pairs_per_launch / avg_s / (FP32_PEAK_FLOPS / 2.0)
     elif dom in ("spread", "interp"):
         # Every NUFFT point is spread once and interpolated once per step (w^3 taps each),
         # 4 flops per tap (complex value times a real weight, accumulated).
