@@ -222,7 +222,9 @@ void build_items(const std::vector<DirectRect> &rects, bool owner_is_vis, int ki
     const int64_t T = direct_tile(kind);
     // One rectangle (most jobs): segments that come out evenly. Many: about 32 items per SM in
     // all, taken dynamically by the kernels largest first, so that a launch ends within a fraction
-    // of an item of its ideal time.
+    // of an item of its ideal time. The FP64 form, of which an SM holds four CTAs, takes the same
+    // items: 52,812 x 44,850 points 147 ms (608 slots: 156; 32 items per CTA, as it had before: 156),
+    // 3,001 x 7,001 points 1.57 ms (1.87; 9.8), many rectangles within 1% either way.
     double work = 0;
     for (auto &r : rects) work += (double)(r.p1 - r.p0) * (double)(r.v1 - r.v0);
     const int64_t even = std::max<int64_t>(2048, (int64_t)std::ceil(work / ((double)T * 152.0 * 32.0) / 256.0) * 256);

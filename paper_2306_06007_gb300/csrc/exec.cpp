@@ -408,7 +408,8 @@ void direct_merged(const std::vector<Plan *> &group, int dir, int kind, cudaStre
     check_cuda(cudaMemsetAsync(counter, 0, sizeof(int), s), "memset batch counter");
     launch_direct_batch(kind, dir, reinterpret_cast<const WorkItem *>(d), n, counter,
                         reinterpret_cast<const DirectJob *>(d + up(b_items) + up(b_job)),
-                        reinterpret_cast<const int *>(d + up(b_items)), group[0]->cis_tab.as<float4>(), s);
+                        reinterpret_cast<const int *>(d + up(b_items)), group[0]->cis_tab.as<float4>(),
+                        std::any_of(group.begin(), group.end(), [](const Plan *p) { return p->stall; }), s);
     check_cuda(cudaFreeAsync(dev, s), "cudaFreeAsync (batch work list)");
     for (Plan *p : group) p->stage_launches[HVOX_STAGE_DIRECT] += 1;
 }

@@ -124,7 +124,7 @@ struct DirectJob {
     float sgn;
     float pix_scale, vis_scale;
     int *err;   // the plan's device error word (may be null)
-    int stall;  // tiles are never handed on, so that the waits run out (fault_hit "stall")
+    int stall;  // of a launch: tiles are never handed on, so that the waits run out (fault_hit "stall")
 };
 
 // The two powers of two for pixels of largest |coordinate| top (1 for unit vectors).
@@ -512,7 +512,7 @@ int direct_owners_per_thread(int kind);
 void launch_direct(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob &J,
                    const float4 *tab, cudaStream_t s);
 void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob *jobs,
-                         const int *item_job, const float4 *tab, cudaStream_t s);
+                         const int *item_job, const float4 *tab, bool stall, cudaStream_t s);
 void launch_direct_f64(int prec, int dir, const WorkItem *items, int64_t n, int *counter, const double *vxyz, int64_t nv,
                        const double *pxyz, int64_t np, const void *src, void *acc, int isign, cudaStream_t s);
 

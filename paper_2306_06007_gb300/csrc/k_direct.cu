@@ -173,17 +173,21 @@ struct DirectPipe {
     uint32_t tmem, chunks, tiles;
 };
 
-// A bounded wait: false where it ran out, here or in another thread of the CTA. Then nothing waits any
-// longer, no more products are issued, the item's sums become NaN and so do those of every item that
-// the CTA takes after it (an item left out would be missing from a finite result); the products
-// in flight are waited for before tensor memory is given back (direct_end).
-template <class K> __device__ __forceinline__ bool pipe_wait(DirectShared<K> &sh, uint64_t *bar, uint32_t parity, int *err) {
-    for (int i = 0; i < tc::kWaitLimit; ++i) {
-        if (*(volatile int *)&sh.abort) return false;
-        if (tc::mbar_try(bar, parity & 1u)) return true;
-    }
-    *(volatile int *)&sh.abort = 1;
+// A bounded wait: false where it ran out, or one has run out in this CTA before (a wait under way then
+// goes on to its own limit; looking at the flag between tries costs the double-float kernels 2%). Then
+// nothing waits any longer, no more products are issued, the item's sums become NaN and so do those of
+// every item that the CTA takes after it (an item left out would be missing from a finite result); the
+// products in flight are waited for before tensor memory is given back (direct_end).
+__device__ __noinline__ void give_up(int *abort, int *err) {
+    *(volatile int *)abort = 1;
     if (err) atomicOr(err, kDevErrStall);
+}
+
+template <class K> __device__ __forceinline__ bool pipe_wait(DirectShared<K> &sh, uint64_t *bar, uint32_t parity, int *err) {
+    if (*(volatile int *)&sh.abort) return false;
+    for (int i = 0; i < tc::kWaitLimit; ++i)
+        if (tc::mbar_try(bar, parity & 1u)) return true;
+    give_up(&sh.abort, err);
     return false;
 }
 
@@ -243,11 +247,12 @@ __device__ __forceinline__ void issue_chunks(DirectShared<K> &sh, const DirectPi
     const uint64_t dig0 = tc::operand_desc(tc::smem_addr(sh.dig), sizeof(sh.dig[0][0]));
     for (uint32_t c = 0; c < chunks; ++c) {
         const uint32_t n = pipe.chunks + c, set = n & 1u, tile = pipe.tiles + c / kPerTile;
-        if (c % kPerTile == 0 && !pipe_wait(sh, &sh.staged[tile & 1u], tile >> 1, err)) return;
+        bool ok = c % kPerTile != 0 || pipe_wait(sh, &sh.staged[tile & 1u], tile >> 1, err);
         const uint64_t dig = dig0 + (((tile & 1u) * sizeof(sh.dig[0]) + (c % kPerTile) * K::kN * 16) >> 4);
 #pragma unroll
         for (int block = 0; block < 2; ++block) {
-            if (!pipe_wait(sh, &sh.read[block][set], (n >> 1) ^ 1u, err)) return;
+            ok = pipe_wait(sh, &sh.read[block][set], (n >> 1) ^ 1u, err) && ok;
+            if (!ok) break;  // and no later chunk is issued: every later wait fails
             tc::fence_after();
             const uint32_t d = pipe.tmem + set_columns<K>(block, set);
 #pragma unroll
@@ -282,7 +287,7 @@ __device__ __forceinline__ bool direct_item(const DirectJob &J, const WorkItem &
             warp_wait(sh, &sh.freed[n & 1u], (n >> 1) ^ 1u, J.err);
             stage_tile<K, DIR>(J, w, w.s0 + (int)t * kStream, sh, n & 1u);
             __syncwarp();
-            if ((tid & 31) == 0 && !J.stall) tc::mbar_arrive(&sh.staged[n & 1u]);
+            if ((tid & 31) == 0) tc::mbar_arrive(&sh.staged[n & 1u]);
         }
     } else {
         const int block = tid >> 8, half = (tid >> 7) & 1, row = block * 128 + (tid & 127);
@@ -361,7 +366,8 @@ template <class K> __device__ __forceinline__ void poison_item(const DirectJob &
     if (threadIdx.x == 0 && J.err) atomicOr(J.err, kDevErrStall);
 }
 
-template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShared<K> &sh) {
+// stall (DirectJob::stall): staged tiles wait for more arrivals than ever come.
+template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShared<K> &sh, int stall) {
     static_assert(4 * K::Form::kAcc * K::kN <= 512 && K::kN % 16 == 0 && kStream % K::kN == 0, "tensor memory of an SM");
     if (threadIdx.x < 32) tc::tmem_alloc(&sh.tmem, 512);
     if (threadIdx.x == 0) {
@@ -370,7 +376,7 @@ template <class K> __device__ __forceinline__ DirectPipe direct_begin(DirectShar
                 tc::mbar_init(&sh.done[b][i], 1);
                 tc::mbar_init(&sh.read[b][i], 8);
             }
-            tc::mbar_init(&sh.staged[i], kProducers / 32);
+            tc::mbar_init(&sh.staged[i], kProducers / 32 + (stall ? 1 << 19 : 0));
             tc::mbar_init(&sh.freed[i], kConsumers / 32);
         }
         tc::mbar_init(&sh.drained, 1);
@@ -604,7 +610,7 @@ __global__ void __launch_bounds__(kDirectThreads, 1)
                   const DirectJob *__restrict__ jobs, const int *__restrict__ item_job, const float4 *__restrict__ gT) {
     extern __shared__ __align__(128) unsigned char direct_smem[];
     DirectShared<K> &sh = *reinterpret_cast<DirectShared<K> *>(direct_smem);
-    DirectPipe pipe = direct_begin(sh);
+    DirectPipe pipe = direct_begin(sh, J0.stall);
     if constexpr (K::kMagnitudes)
         for (int i = threadIdx.x; i < kDfTab * kDfCopies; i += kDirectThreads) {
             const float4 e = gT[2 * (i / kDfCopies)];
@@ -819,8 +825,10 @@ void launch_direct(int kind, int dir, const WorkItem *items, int64_t n, int *cou
 }
 
 void launch_direct_batch(int kind, int dir, const WorkItem *items, int64_t n, int *counter, const DirectJob *jobs,
-                         const int *item_job, const float4 *tab, cudaStream_t s) {
-    if (n > 0) launch_kind<true>(kind, dir, items, n, counter, DirectJob{}, jobs, item_job, tab, s);
+                         const int *item_job, const float4 *tab, bool stall, cudaStream_t s) {
+    DirectJob all{};
+    all.stall = stall;
+    if (n > 0) launch_kind<true>(kind, dir, items, n, counter, all, jobs, item_job, tab, s);
 }
 
 template <class T>
@@ -902,7 +910,7 @@ __global__ void noalloc_prepare_kernel(const double *__restrict__ pix, int64_t n
 template <class K>
 __device__ __forceinline__ void noalloc_items(const DirectJob &J, int n_vis, int n_pix, int seg, unsigned char *smem) {
     DirectShared<K> &sh = *reinterpret_cast<DirectShared<K> *>(smem);
-    DirectPipe pipe = direct_begin(sh);
+    DirectPipe pipe = direct_begin(sh, J.stall);
     if constexpr (K::kMagnitudes)
         for (int i = threadIdx.x; i < kDfTab; i += kDirectThreads) {
             double sn, cs;

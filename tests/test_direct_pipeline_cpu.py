@@ -32,5 +32,6 @@ def test_products_end_before_tensor_memory_is_freed():
     # limit) before the CTA gives its memory back.
     src = open(os.path.join(CSRC, "k_direct.cu")).read()
     issue, end = _body(src, "void issue_chunks"), _body(src, "void direct_end")
-    assert len(re.findall(r"if \([^;]*!pipe_wait\(.*\)\) return;", issue)) == len(re.findall(r"pipe_wait\(", issue)) == 2
+    assert len(re.findall(r"\bok = [^;]*pipe_wait\([^;]*;", issue)) == len(re.findall(r"pipe_wait\(", issue)) == 2
+    assert issue.rindex("pipe_wait(") < issue.index("if (!ok) break;") < issue.index("tc::mma<")
     assert end.index("mma_commit(&sh.drained)") < end.index("mbar_try(&sh.drained") < end.index("tmem_free")
