@@ -603,8 +603,10 @@ bool cfft_factor(int n, CfftDev &d) {
 }
 
 // Rows and columns of these lengths fit a CTA, the y columns in tiles of whole 32-byte sectors
-// (4 or more); longer ones stay with cuFFT. Indices inside a CTA stay below 2^16, where the
-// divisions by multiplication are exact.
+// (4 or more): no y length above 4,096, and below that not those whose stage in between would need
+// more than 1,024 threads (1,750 = 5 5 14 5, 2,000, 2,058, 2,430, ...: its radix under n / 256). The rest
+// stays with cuFFT, and takes every grid of its plan along (Plan::cf_grids). Indices inside a CTA stay
+// below 2^16, where the divisions by multiplication are exact.
 bool cfft_supported(const int64_t n2[3]) {
     CfftDev d[3];
     for (int k = 0; k < 3; ++k)

@@ -90,7 +90,7 @@ template <int SG> __device__ __forceinline__ void twiddle(const float4 *__restri
 // the R outputs to (j / Ns) Ns R + k + q Ns. q k span < n, so the table index needs no wrap.
 // The sign SG of the exponent is a template parameter: its flips fold into the operands.
 // ld(e, t) reads element e of sequence t, st(e, t, v) writes it: shared memory between
-// stages; the grid itself in the first and the last stage of a z-column pass.
+// stages, the grid itself in the first and the last stage of a pass.
 template <int R, int TX, int SG, class Ld, class St>
 __device__ __forceinline__ void stage(Ld ld, St st, const DfftDev &d, int Ns, unsigned magic) {
     const int n = d.n, m = n / R, span = n / (Ns * R);

@@ -11,7 +11,10 @@
 //    hardware sin/cos approximations, FP32 accumulation;
 //  * double-float path (eps < 1e-6): exp(j 2 pi f) as the hi parts of a 1024-entry table of
 //    exp(j 2 pi m / 1024) plus a lo part (the table's lo parts and a short series in the
-//    remainder, in plain float; error ~1e-10); sums in double-float arithmetic (Dekker 1971);
+//    remainder, in plain float); sums in double-float arithmetic (Dekker 1971). A term is off by
+//    1.0e-10 rms and 5.7e-10 at most (restated on the CPU; 5.3e-11 and 2.8e-10 with 2,048 entries,
+//    which do not fit eightfold in shared memory) and the sums add nothing to it: rel. l2 of V within
+//    1,000 wavelengths 1.3e-10 for 16, 64 and 4,000 pixels (on the FP32 pipes 1.0e-10, 1.45e-10, 2.5e-10);
 //  * wide path: the double-float path on the values of an FP32 plan whose |p_d r_d| exceed 2^28
 //    turns (the reach of the FP32 digits);
 //  * plain path: everything in FP64 (the reference form the optimised paths replace; also, on the
@@ -21,9 +24,9 @@
 // the 20 that 32 pairs take), in double-float the FMA pipe (60% busy), the shared-memory pipe (63%)
 // and issue (64%) together. FMAs and adds go two to an instruction (f32x2) over two columns or over
 // a sum's two parts: they take the FMA pipe as long as two scalar ones but half the issue slots.
-// Measured on one GB300 over 52,812 pixels x 1,435,200 baselines, pairs/s: FP32 1.16e12 with the
-// phase on the FP32 pipes, 1.95e12 with it on the tensor cores, 2.05e12 with f32x2; double-float
-// 4.7e11, 7.1e11 and 8.2e11.
+// Measured on one GB300 over the 52,812 pixels x 1,435,200 baselines of the LOFAR-like step, all direct,
+// both directions, pairs/s: FP32 2.00e12 and double-float 7.9e11; with the phase on the FP32 pipes 1.16e12 and
+// 4.7e11, on the tensor cores but without f32x2 1.95e12 and 7.1e11.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>

@@ -183,10 +183,11 @@ CostModel default_cost_model(int prec, bool plain, int w, bool z2z_fft) {
         // large launch of the SKA-Low-like benchmark line (2.9e12 pairs per launch), since
         // the calibration workloads have almost no direct work.
         // These are the rates of the stored fits. The kernels are faster by now (direct pairs
-        // 2.05e12/s at FP32 and 8.2e11/s in double-float, FFTs 1.2 to 2 times), and direct sums and
-        // FFTs by similar factors; with the new direct rate alone the dense core goes from 1 to 21
-        // sub-problems on a near tie (12.43 against 12.35 ms modelled) and its small FFT batches,
-        // which the model does not see, took 12.9 ms instead of 7.9.
+        // 2.0e12/s at FP32 and 7.9e11/s in double-float, FFTs 1.2 to 2 times), and direct sums and
+        // FFTs by similar factors. The new direct rate alone was tried while FP32 grids still went
+        // through cuFFT: the dense core went from 1 to 21 sub-problems on a near tie (12.43 against
+        // 12.35 ms modelled), whose small FFT batches the model does not see (its FFTs 7.9 -> 12.9 ms).
+        // With the library's own FFT (7.0 ms for the one sub-problem) it has not been measured again.
         m.direct_pair = 1.0 / 1.17e12;
         m.scatter_smem = 1.0 / 6.3e11;
         m.scatter_global = 1.0 / 2.4e11;
